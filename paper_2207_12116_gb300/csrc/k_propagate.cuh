@@ -35,6 +35,11 @@ struct PropArgs {
   uint32_t tlev_bytes;  // table_global, in place: temporal levels staged per CTA (0: none)
   uint32_t off_tlev;    // their offset in the image
   int levels;           // temporal levels: bit 0 staged tables, bit 1 global ones
+  // mask form only: the caller's variables' places in the store, four copies
+  // of map_stride entries, copy h readable 16 bytes at a time from variable h
+  const uint32_t* map;
+  int map_stride;
+  uint32_t slot_bytes;  // shared memory of a team (mask form)
 };
 
 // Per-team scalars of k_propagate (shared memory).

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <climits>
 #include <cmath>
@@ -22,12 +23,15 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <string>
 #include <unordered_map>
 #include <vector>
 
 #include "../../include/pccp.h"
 #include "pccp_device.cuh"
 #include "k_propagate.cuh"
+#include "mask_device.cuh"
+#include "k_propagate_mask.cuh"
 #include "k_solve_eps.cuh"
 #include "policy_train.cuh"
 
@@ -100,6 +104,7 @@ struct SolveArgs {
   uint32_t slot_bytes;
   uint32_t off_track, off_x, off_stack, off_store;  // byte offsets inside a slot
   int levels;  // temporal levels: bit 0 with tables in shared memory, bit 1 in global memory
+  uint32_t pol_bytes;  // k_solve_mask: the staged network, before the slots
 };
 
 // Broadcast slots of one team's search.  Each slot has one writer (thread 0)
@@ -435,11 +440,17 @@ __global__ void __launch_bounds__(1024) k_solve_slots(SolveArgs a) {
   }
   int2* stack = reinterpret_cast<int2*>(slot + a.off_stack);
   uint32_t parity = 0;
-  for (;;) {
+  // the first model by position, CTA by CTA, so that models spread over the
+  // SMs before teams share one; the others from the counter
+  const int n_teams = static_cast<int>(gridDim.x) * a.teams;
+  int q = static_cast<int>(blockIdx.x) + team_id * static_cast<int>(gridDim.x);
+  for (bool first = true;; first = false) {
     team_bar(tm.bar, tm.nthr);  // the previous model is done (first pass: mbarrier ready)
-    if (tm.tid == 0) sc->next = atomicAdd(a.counter, 1);
-    team_bar(tm.bar, tm.nthr);
-    const int q = sc->next;
+    if (!first) {
+      if (tm.tid == 0) sc->next = n_teams + atomicAdd(a.counter, 1);
+      team_bar(tm.bar, tm.nthr);
+      q = sc->next;
+    }
     if (q >= a.n_inst) break;
     const InstanceDesc d = a.inst[q];
     InstanceResult* out = &a.res[d.index];
@@ -497,6 +508,7 @@ __global__ void __launch_bounds__(1024) k_solve_slots(SolveArgs a) {
   }
 }
 
+#include "mask_search.inc"
 #include "k_search_queue.inc"
 
 // -------------------------------------------------------------- host model
@@ -531,6 +543,10 @@ const PolicyDev* policy_dev(const pccp_policy* p);
 
 struct HostPipe;
 
+namespace {
+#include "mask_form.inc"
+}  // namespace
+
 struct pccp_model {
   int device;
   int32_t n_vars, n_t, n_rf, n_lin, n_terms, n_branch, objective;
@@ -547,6 +563,7 @@ struct pccp_model {
   uint32_t tlev_bytes;    // their section, the last tlev_bytes of the core prefix
   uint8_t* d_mem;    // image, then root int2[n_vars]
   int2* d_root;
+  MaskForm mask;     // the mask form, when the model has one
   HostPipe* pipe = nullptr;  // pccp_propagate_host's streams and slots (lazy)
   std::mutex pipe_mu;               // one host-memory propagation at a time
 };
@@ -1341,7 +1358,67 @@ struct PropPlan {
   uint32_t tlev_bytes;  // rows read in place: the temporal levels staged per CTA (0: none)
   int team, teams, grid, max_grid;
   size_t smem;
+  bool mask;  // k_propagate_mask on the model's mask form
+  uint32_t slot_bytes;
 };
+
+// The mask form's plan; p->mask stays false when some team does not fit (the
+// general kernels then say what does).
+int plan_propagate_mask(const pccp_model* m, int32_t n_stores, const pccp_launch_config* cfg,
+                        int smem_max, int sms, PropPlan* p) {
+  const MaskForm& f = m->mask;
+  const size_t per_team = align16(16 + 4 * static_cast<size_t>(mask_ctrl_words(f.n_words)) +
+                                  static_cast<size_t>(f.n_slots) * sizeof(int2));
+  const size_t base = static_cast<size_t>(f.image_bytes) + 16;
+  int team = 64, teams = 0;
+  if (cfg && cfg->team_threads > 0) {
+    team = cfg->team_threads;
+  } else {
+    // the most warps a store that still give every warp of the GPU about two
+    // and a half (enough stores in turn that a hard one does not hold up the
+    // end), at least two (the two directions of the temporal levels), at most
+    // one a pair of words.  Measured, us with 2 / 4 / 8 / 16 / 32 warps a store:
+    // 10,000 stores of 30 tasks 110 / 115 / 157 / 237 / 408, 777 of 60 170 /
+    // 114 / 114 / 99 / 112, 1,216 of 120 319 / 184 / 191 / 195 / 199, 152 of
+    // 120 305 / 181 / 135 / 106 / 84 (each about 40 us of it call overhead)
+    const int pairs = (f.n_words + 1) / 2;
+    while (team < 1024 && team / 32 < pairs &&
+           2ll * n_stores * (team / 32) <= 5ll * sms * 16)
+      team *= 2;
+  }
+  if (cfg && cfg->teams_per_cta > 0) teams = cfg->teams_per_cta;
+  if (teams == 0) {  // 32 warps an SM; fewer when there is a store for no more teams
+    teams = std::min(1024 / team, team == 32 ? 32 : 16);
+    teams = std::max(1, std::min(teams, (n_stores + sms - 1) / sms));
+  }
+  if (team * teams > 1024 || base + per_team > static_cast<size_t>(smem_max)) return PCCP_OK;
+  const int fit = static_cast<int>((static_cast<size_t>(smem_max) - base) / per_team);
+  if (teams > fit) {
+    if (cfg && cfg->teams_per_cta > 0) return PCCP_OK;
+    teams = fit;
+  }
+  const size_t smem = base + static_cast<size_t>(teams) * per_team;
+  const auto kern = team == 32 ? k_propagate_mask<true, 1024, 1> : k_propagate_mask<false, 1024, 1>;
+  PCCP_CUDA(allow_smem(reinterpret_cast<const void*>(kern), smem));
+  int per_sm = 0;
+  PCCP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, teams * team, smem));
+  if (per_sm < 1) return PCCP_OK;
+  if (cfg && cfg->ctas_per_sm > 0) per_sm = std::min(per_sm, static_cast<int>(cfg->ctas_per_sm));
+  const int want = (n_stores + teams - 1) / teams;
+  p->kern = kern;
+  p->table_global = false;
+  p->copy_bytes = f.image_bytes;
+  p->stages = 0;
+  p->tlev_bytes = 0;
+  p->team = team;
+  p->teams = teams;
+  p->max_grid = sms * per_sm;
+  p->grid = std::max(1, std::min(want, p->max_grid));
+  p->smem = smem;
+  p->mask = true;
+  p->slot_bytes = static_cast<uint32_t>(per_team);
+  return PCCP_OK;
+}
 
 int plan_propagate(const pccp_model* m, int32_t n_stores, const pccp_launch_config* cfg,
                    PropPlan* p) {
@@ -1350,6 +1427,13 @@ int plan_propagate(const pccp_model* m, int32_t n_stores, const pccp_launch_conf
   if (smem_max <= 0 || sms <= 0) return PCCP_ERR_CUDA;
   int team = (cfg && cfg->team_threads > 0) ? cfg->team_threads : 128;
   if (team % 32 != 0 || team > 1024) return PCCP_ERR_INVALID;
+  if (cfg && cfg->teams_per_cta > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
+  p->mask = false;
+  p->slot_bytes = 0u;
+  if (m->mask.ok && !(cfg && (cfg->skip_stable > 0 || cfg->stream_table > 0))) {
+    const int rc = plan_propagate_mask(m, n_stores, cfg, smem_max, sms, p);
+    if (rc != PCCP_OK || p->mask) return rc;
+  }
   const size_t per_team = sizeof(PropCtrl) + 4 * ((track_words(m->n_vars, m->n_lin) + 3) & ~3) +
                           static_cast<size_t>(m->n_slots) * sizeof(int2);
   // the table lives in shared memory when it fits beside one team's store
@@ -1368,7 +1452,6 @@ int plan_propagate(const pccp_model* m, int32_t n_stores, const pccp_launch_conf
   // to 64 registers; measured ahead of 4 x 128 with three CTAs per SM and a
   // 40-register cap)
   int teams = (cfg && cfg->teams_per_cta > 0) ? cfg->teams_per_cta : 8;
-  if (teams > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
   teams = std::min({teams, fit, 1024 / team});
   if (cfg && cfg->teams_per_cta > 0 && teams < cfg->teams_per_cta) return PCCP_ERR_SMEM;
   if (teams < 1) return PCCP_ERR_SMEM;
@@ -1429,8 +1512,10 @@ int launch_propagate(const pccp_model* m, const PropPlan& plan, int32_t n_stores
                      int32_t* ub, int32_t* status, int32_t* iterations, int32_t* work,
                      const pccp_launch_config* cfg, int* counter, cudaStream_t s) {
   PropArgs a;
-  a.image = m->d_mem;
-  a.root = m->d_root;
+  a.image = plan.mask ? m->mask.d_mem : m->d_mem;
+  a.root = plan.mask ? m->mask.d_root : m->d_root;
+  a.map = m->mask.d_map;
+  a.map_stride = m->mask.map_stride;
   a.lb = lb;
   a.ub = ub;
   a.status = status;
@@ -1438,12 +1523,14 @@ int launch_propagate(const pccp_model* m, const PropPlan& plan, int32_t n_stores
   a.counter = counter;
   a.image_bytes = plan.table_global ? m->image_bytes : plan.copy_bytes;
   a.n_vars = m->n_vars;
-  a.n_slots = m->n_slots;
+  a.n_slots = plan.mask ? m->mask.n_slots : m->n_slots;
   a.n_stores = n_stores;
   a.team_size = plan.team;
   a.teams = plan.teams;
   a.max_iter = (cfg && cfg->max_iterations > 0) ? cfg->max_iterations : m->max_iter;
-  a.track_words = track_words(m->n_vars, m->n_lin);
+  a.track_words = plan.mask ? mask_ctrl_words(m->mask.n_words)
+                            : track_words(m->n_vars, m->n_lin);
+  a.slot_bytes = plan.mask ? plan.slot_bytes : 0u;
   a.work = work;
   a.table_global = plan.table_global ? 1 : 0;
   a.stream_stages = plan.stages;
@@ -1465,6 +1552,8 @@ struct BatchPlan {
   size_t smem;           // dynamic shared memory per CTA
   uint32_t slot_bytes, off_track, off_x, off_stack, off_store;
   int xw, max_tw, max_vars, stages;
+  bool mask;           // k_solve_mask on the models' mask forms
+  uint32_t pol_bytes;  // k_solve_mask: shared memory before the slots
 };
 
 // Shared memory a model needs in a slot whose store starts at off_store:
@@ -1483,12 +1572,110 @@ uint32_t slot_need_global(const pccp_model* m, uint32_t off_store, uint32_t room
   return m->n_tlev > 0 && with <= room ? with : st_end;
 }
 
+// Slot bytes of a model in mask form whose store starts at off_store.
+uint32_t slot_need_mask(const pccp_model* m, uint32_t off_store) {
+  const uint32_t st_end = off_store + 8u * static_cast<uint32_t>(m->mask.n_slots);
+  return ((st_end + 127u) & ~127u) + m->mask.core_bytes;
+}
+
+// The k_solve_mask instantiation of a strategy for teams of `team` threads.
+SolveKernel mask_kernel(bool learned, int team) {
+  if (team == 32) return learned ? k_solve_mask<true, true> : k_solve_mask<true, false>;
+  return learned ? k_solve_mask<false, true> : k_solve_mask<false, false>;
+}
+
+// Plans a batched search of models that all have a mask form; p->mask stays
+// false when some model has none or does not fit, when the caller asks for what
+// only the general kernels have (change tracking, streamed tables), or for
+// more than 512 threads a CTA.
+int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
+                    bool any_strategy, int smem_max, int sms, BatchPlan* p) {
+  if (o->skip_stable > 0 || o->stream_table > 0) return PCCP_OK;
+  int32_t max_branch = 0, max_tw = 0, max_words = 0, max_rows = 0, max_dec = 2;
+  for (int32_t i = 0; i < n; ++i) {
+    const pccp_model* m = models[i];
+    if (!m->mask.ok) return PCCP_OK;
+    max_branch = std::max(max_branch, m->n_branch);
+    max_tw = std::max(max_tw, mask_search_words(m->mask.n_words, m->mask.bit0));
+    max_words = std::max(max_words, m->mask.n_words);
+    max_rows = std::max(max_rows, m->n_t + m->n_rf + m->n_lin);
+    max_dec = std::max(max_dec, m->max_decisions);
+  }
+  const bool learned = o->strategy == PCCP_LEARNED;
+  p->xw = any_strategy ? 24 * ((max_branch + 15) & ~15) : policy_x_words(o, max_branch);
+  p->max_depth = max_dec;
+  p->off_track = static_cast<uint32_t>(align16(16 + sizeof(SearchCtrl)));
+  p->off_x = p->off_track + 4u * static_cast<uint32_t>((max_tw + 3) & ~3);
+  p->off_stack = static_cast<uint32_t>(align16(p->off_x + 4u * static_cast<uint32_t>(p->xw)));
+  p->off_store = static_cast<uint32_t>(
+      align16(p->off_stack + sizeof(int2) * static_cast<size_t>(p->max_depth)));
+  p->pol_bytes = learned || any_strategy
+                     ? static_cast<uint32_t>((sizeof(PolicyDev) + 127u) & ~static_cast<size_t>(127))
+                     : 0u;
+  uint32_t need = 0;
+  int64_t ring = 0;  // every depth of the deepest path
+  for (int32_t i = 0; i < n; ++i) {
+    const pccp_model* m = models[i];
+    need = std::max(need, slot_need_mask(m, p->off_store));
+    ring = std::max(ring, static_cast<int64_t>(m->max_decisions) *
+                              mask_ring_entry(m->mask.n_slots, m->mask.n_words));
+  }
+  auto room_of = [&](int teams) {
+    return static_cast<uint32_t>((smem_max - static_cast<int>(p->pol_bytes)) / teams) & ~127u;
+  };
+  // one team an SM until there are more models than SMs
+  int teams = o->teams_per_cta;
+  if (teams == 0) {
+    teams = std::max(1, std::min({8, 512 / std::max(o->threads, 32), (n + sms - 1) / sms}));
+    while (teams > 1 && need > room_of(teams)) --teams;
+  }
+  int team = o->threads;
+  if (team == 0 && o->props_per_thread > 0)
+    team = std::min(512 / teams, std::max(32, ((max_rows + o->props_per_thread - 1) /
+                                                   o->props_per_thread + 31) & ~31));
+  if (team == 0) {
+    // a warp per sixteen words of Booleans: a node runs few of them, and a
+    // barrier costs more with more warps (256 30-60-task models x 500 nodes, two
+    // teams an SM of 64 / 128 / 256 threads: 12.7 / 9.9 / 9.6 ms; 64 60-task models,
+    // learned, one team of 128 / 256 / 512: 3.8 / 3.1 / 3.0 ms; one 8-task model of
+    // 2,559 nodes, 32 / 64 / 128: 12.6 / 13.4 / 13.4 ms)
+    int w = 1;
+    while (64 * w * teams <= 512 && 16 * w < max_words) w *= 2;
+    team = 32 * w;
+  }
+  if (team < 32 || team * teams > 512 || need > room_of(teams)) return PCCP_OK;
+  p->slots = true;
+  p->stages = 0;
+  p->max_tw = max_tw;
+  p->max_vars = 0;
+  p->kern = mask_kernel(learned, team);
+  p->slot_bytes = static_cast<uint32_t>(
+      std::min<int64_t>(room_of(teams), (need + ring + 16 + 127) & ~static_cast<int64_t>(127)));
+  p->team = team;
+  p->teams = teams;
+  p->smem = p->pol_bytes + static_cast<size_t>(teams) * p->slot_bytes;
+  int per_sm = 1 << 30;
+  for (int k = 0; k < 2; ++k) {
+    if (!any_strategy && learned != (k == 1)) continue;
+    const SolveKernel kern = mask_kernel(k == 1, team);
+    PCCP_CUDA(allow_smem(reinterpret_cast<const void*>(kern), p->smem));
+    int occ = 0;
+    PCCP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, team * teams, p->smem));
+    per_sm = std::min(per_sm, occ);
+  }
+  if (per_sm < 1) return PCCP_OK;
+  p->grid = std::max(1, std::min(static_cast<int>(n), sms * per_sm));
+  if (o->blocks > 0) p->grid = std::min(p->grid, static_cast<int>(o->blocks));
+  p->mask = true;
+  return PCCP_OK;
+}
+
 // Plans a batched search.  any_strategy: room for the learned strategy's
 // feature rows and an occupancy valid for every strategy's kernel (a batch
 // planned once for later searches).  Returns SMEM when some store does not
 // fit a slot.
 int plan_batch(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
-               bool any_strategy, BatchPlan* p) {
+               bool any_strategy, BatchPlan* p, bool allow_mask = true) {
   const int smem_max = max_dyn_smem();
   const int sms = sm_count();
   if (smem_max <= 0 || sms <= 0) return PCCP_ERR_CUDA;
@@ -1507,6 +1694,12 @@ int plan_batch(const pccp_model* const* models, int32_t n, const pccp_solve_opts
   if (o->threads < 0 || o->threads % 32 != 0 || o->threads > 1024) return PCCP_ERR_INVALID;
   if (o->teams_per_cta < 0 || o->teams_per_cta > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
   if (o->props_per_thread < 0) return PCCP_ERR_INVALID;
+  p->mask = false;
+  p->pol_bytes = 0u;
+  if (allow_mask) {
+    const int rc = plan_batch_mask(models, n, o, any_strategy, smem_max, sms, p);
+    if (rc != PCCP_OK || p->mask) return rc;
+  }
   p->xw = any_strategy ? 24 * ((max_branch + 15) & ~15) : policy_x_words(o, max_branch);
   p->max_tw = max_tw;
   p->max_vars = max_vars;
@@ -1633,11 +1826,11 @@ std::vector<int32_t> batch_order(const pccp_model* const* models, int32_t n) {
 }
 
 // Descriptor of model i (position `index` in the caller's list).
-InstanceDesc instance_desc(const pccp_model* m, int32_t index, int32_t witness_off) {
+InstanceDesc instance_desc(const pccp_model* m, int32_t index, int32_t witness_off, bool mask) {
   InstanceDesc d;
-  d.image = m->d_mem;
-  d.root = m->d_root;
-  d.image_bytes = m->image_bytes;
+  d.image = mask ? m->mask.d_mem : m->d_mem;
+  d.root = mask ? m->mask.d_root : m->d_root;
+  d.image_bytes = mask ? m->mask.core_bytes : m->image_bytes;
   d.n_vars = m->n_vars;
   d.witness_off = witness_off;
   d.n_branch = m->n_branch;
@@ -1672,6 +1865,7 @@ SolveArgs batch_args(const BatchPlan& p, const pccp_solve_opts* o, int32_t n) {
   a.off_x = p.off_x;
   a.off_stack = p.off_stack;
   a.off_store = p.off_store;
+  a.pol_bytes = p.pol_bytes;
   return a;
 }
 
@@ -1705,11 +1899,12 @@ int pccp_model_create(const pccp_model_desc* desc_user, pccp_model** out) {
   const int32_t nv_user = desc_user->n_vars > 0 ? desc_user->n_vars : 0;
   // Booleans kept as bits when the model allows it (bit_vars) and either the
   // caller asks for it or an interval store would exceed kBitStoreMinBytes
-  std::vector<char> bits;
+  std::vector<char> bits, mask_bits;
   int32_t n_bits = 0;
   if (desc_user->bool_store >= 0) {
     bits = bit_vars(desc_user);
     for (char b : bits) n_bits += b ? 1 : 0;
+    if (n_bits > 0) mask_bits = bits;
     // by default only where an interval store could not fit in shared memory
     // at all (the model would be refused): bits cost an extraction per
     // Boolean read and are read only by the global-table kernels, which
@@ -1860,6 +2055,14 @@ int pccp_model_create(const pccp_model_desc* desc_user, pccp_model** out) {
     delete m;
     return PCCP_ERR_CUDA;
   }
+  if (!mask_bits.empty()) {  // without it the model runs on the primary table
+    MaskPacked mp;
+    if (pack_mask(desc_user, mask_bits, p, iof, &mp) && !mask_upload(mp, &m->mask)) {
+      (void)cudaGetLastError();
+      cudaFree(m->mask.d_mem);
+      m->mask = MaskForm();
+    }
+  }
   *out = m;
   return PCCP_OK;
 }
@@ -1871,6 +2074,7 @@ void pccp_model_destroy(pccp_model* m) {
   cudaSetDevice(m->device);
   cudaDeviceSynchronize();
   host_pipe_free(m->pipe);
+  cudaFree(m->mask.d_mem);
   cudaFree(m->d_mem);
   if (prev >= 0) cudaSetDevice(prev);
   delete m;
@@ -1909,6 +2113,8 @@ int pccp_propagate_ex(const pccp_model* m, int32_t n_stores, int32_t* lb, int32_
   if (rc != PCCP_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int* counter = nullptr;
+  if (plan.mask && n_stores <= plan.grid * plan.teams)  // a store per team at most: none is taken
+    return launch_propagate(m, plan, n_stores, lb, ub, status, iterations, work, cfg, nullptr, s);
   PCCP_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&counter), sizeof(int), s));
   PCCP_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), s));
   rc = launch_propagate(m, plan, n_stores, lb, ub, status, iterations, work, cfg, counter, s);
@@ -1956,7 +2162,8 @@ int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
   }
   const std::vector<int32_t> ord = batch_order(models, n_models);
   for (int32_t q = 0; q < n_models; ++q)
-    desc[q] = instance_desc(models[ord[q]], ord[q], woff[ord[q]]);
+    desc[q] = instance_desc(models[ord[q]], ord[q], woff[ord[q]],
+                            plan.mask);
   const int n_teams = plan.grid * plan.teams;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -2377,7 +2584,7 @@ int plan_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opts
     pccp_solve_opts q = *o;
     if (q.threads == 0 && q.props_per_thread == 0) q.threads = default_team(max_rows, 256);
     BatchPlan bp;
-    const int rc = plan_batch(models, n, &q, false, &bp);
+    const int rc = plan_batch(models, n, &q, false, &bp, false);
     if (rc != PCCP_OK) return rc;
     if (!bp.slots) return PCCP_ERR_INVALID;  // streaming is not offered here
     // the same choices with this kernel's control block
@@ -2511,7 +2718,7 @@ int solve_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opt
     woff[i] = static_cast<int32_t>(wit_total);
     wit_total += models[i]->n_vars;
     if (wit_total > INT32_MAX) return PCCP_ERR_INVALID;
-    desc[i] = instance_desc(models[i], i, woff[i]);
+    desc[i] = instance_desc(models[i], i, woff[i], false);
   }
   const size_t per_item = static_cast<size_t>(plan.max_len) * sizeof(int2);
   const size_t cap = queue_cap(n, n_teams, plan.max_len);
@@ -2605,7 +2812,7 @@ int pccp_solve(const pccp_model* m, const pccp_solve_opts* opts, pccp_result* re
     return solve_queue(one, 1, opts, result, static_cast<cudaStream_t>(stream));
   }
   pccp_solve_opts o = *opts;
-  if (o.threads <= 0) o.threads = 512;
+  if (o.threads <= 0 && !(m->mask.ok && o.skip_stable <= 0 && o.stream_table <= 0)) o.threads = 512;
   o.teams_per_cta = 1;  // one model: one team
   const pccp_model* one[1] = {m};
   return pccp_solve_batch(one, 1, &o, result, stream);

@@ -19,7 +19,7 @@ namespace pccp {
 
 enum : int { kFixpoint = 0, kFailed = 1, kError = 2 };
 
-// Header at the start of the packed table image (128 bytes).  The image is
+// Header at the start of the packed table image (256 bytes).  The image is
 // copied verbatim into shared memory, so every offset is relative to its start
 // and 16-byte aligned.
 struct TableHeader {
@@ -43,8 +43,20 @@ struct TableHeader {
   // [n_tlev + 1] at off_tlev, then (16-byte aligned) the rows grouped by the
   // level of x, the length of the longest chain of rows ending at x
   int32_t off_tlev, n_tlev;
+  // mask form (mask_device.cuh; mask = 0: this image is not one): the root in
+  // the store layout, word descriptors, word patterns, mask rows and their
+  // coefficient planes (n_pq quads of planes per word)
+  int32_t mask, off_rs, off_wd, n_wd, off_wp, off_mr, n_mr, off_mp, n_pq;
+  int32_t one_word;  // every mask row has one word and one quad of planes
+  int32_t off_rl;    // root lower bounds of the caller's Booleans as bits, four copies
+  int32_t rl_words;  // words of a copy
+  int32_t off_rank;  // uint16 per word of the store: its descriptor, 0xffff none
+  // searches: n_unit units of each interval variable (0: none), the cross units
+  // and their patterns, the longest paths of the temporal rows (dist_pitch 0: none)
+  int32_t off_unit, n_unit, off_xu, off_xpat, off_dist, dist_pitch;
+  int32_t pad[13];
 };
-static_assert(sizeof(TableHeader) == 128, "header must be 128 bytes");
+static_assert(sizeof(TableHeader) == 256, "header must be 256 bytes");
 
 // Streamed tables.  When a table does not fit in shared memory beside a store,
 // a sweep brings its rows in as a cyclic sequence of segments of at most

@@ -99,6 +99,13 @@ __device__ __forceinline__ void write_features(uint32_t* row, int k, int2 D, int
 // (mlp_row_score), so the result does not depend on how many warps shared
 // the tiles.  Kept out of line so its 40-odd live registers do not raise
 // the register count of the propagation loop.
+// kShared: the network is in shared memory.
+template <bool kShared, class T>
+__device__ __forceinline__ T pol_load(const T* p) {
+  return kShared ? *p : __ldg(p);
+}
+
+template <bool kShared>
 __device__ __noinline__ void mlp_score_tiles(const PolicyDev* __restrict__ pol,
                                              const uint32_t* X, int c, int j0, int j1,
                                              float* part) {
@@ -110,11 +117,11 @@ __device__ __noinline__ void mlp_score_tiles(const PolicyDev* __restrict__ pol,
 #pragma unroll
   for (int kk = 0; kk < 8; ++kk) {
     float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-    mma_16816(d0, a1, __ldg(&pol->w1[2 * kk][lane]));
-    mma_16816(d1, a1, __ldg(&pol->w1[2 * kk + 1][lane]));
+    mma_16816(d0, a1, pol_load<kShared>(&pol->w1[2 * kk][lane]));
+    mma_16816(d1, a1, pol_load<kShared>(&pol->w1[2 * kk + 1][lane]));
     const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-    const float b00 = __ldg(&pol->b1[c0]), b01 = __ldg(&pol->b1[c0 + 1]);
-    const float b10 = __ldg(&pol->b1[c1]), b11 = __ldg(&pol->b1[c1 + 1]);
+    const float b00 = pol_load<kShared>(&pol->b1[c0]), b01 = pol_load<kShared>(&pol->b1[c0 + 1]);
+    const float b10 = pol_load<kShared>(&pol->b1[c1]), b11 = pol_load<kShared>(&pol->b1[c1 + 1]);
     a2[kk][0] = pack_bf16x2(fmaxf(d0[0] + b00, 0.f), fmaxf(d0[1] + b01, 0.f));
     a2[kk][1] = pack_bf16x2(fmaxf(d0[2] + b00, 0.f), fmaxf(d0[3] + b01, 0.f));
     a2[kk][2] = pack_bf16x2(fmaxf(d1[0] + b10, 0.f), fmaxf(d1[1] + b11, 0.f));
@@ -124,10 +131,10 @@ __device__ __noinline__ void mlp_score_tiles(const PolicyDev* __restrict__ pol,
   for (int j = j0; j < j1; ++j) {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) mma_16816(acc, a2[kk], __ldg(&pol->w2[kk][j][lane]));
+    for (int kk = 0; kk < 8; ++kk) mma_16816(acc, a2[kk], pol_load<kShared>(&pol->w2[kk][j][lane]));
     const int c0 = 8 * j + 2 * t;
-    const float bb0 = __ldg(&pol->b2[c0]), bb1 = __ldg(&pol->b2[c0 + 1]);
-    const float w0 = __ldg(&pol->w3[c0]), w1 = __ldg(&pol->w3[c0 + 1]);
+    const float bb0 = pol_load<kShared>(&pol->b2[c0]), bb1 = pol_load<kShared>(&pol->b2[c0 + 1]);
+    const float w0 = pol_load<kShared>(&pol->w3[c0]), w1 = pol_load<kShared>(&pol->w3[c0 + 1]);
     float p_lo = fmaxf(acc[0] + bb0, 0.f) * w0 + fmaxf(acc[1] + bb1, 0.f) * w1;
     float p_hi = fmaxf(acc[2] + bb0, 0.f) * w0 + fmaxf(acc[3] + bb1, 0.f) * w1;
     p_lo += __shfl_xor_sync(0xffffffffu, p_lo, 1);
@@ -142,12 +149,13 @@ __device__ __noinline__ void mlp_score_tiles(const PolicyDev* __restrict__ pol,
 }
 
 // Score of row `row` (0..15) of a chunk from its 16 tile parts, in tile order.
+template <bool kShared>
 __device__ __forceinline__ float mlp_row_score(const PolicyDev* __restrict__ pol,
                                                const float* part, int row) {
   float s = 0.f;
 #pragma unroll
   for (int j = 0; j < 16; ++j) s += part[16 * j + row];
-  return s + __ldg(&pol->b3);
+  return s + pol_load<kShared>(&pol->b3);
 }
 
 // Order-preserving map of a float score to an unsigned integer.
@@ -171,6 +179,7 @@ __device__ __forceinline__ unsigned long long learned_key(float s, int k) {
 // keys to *sel in the minimum form of the plain strategies (~learned_key:
 // its low 32 bits are the branch index).  Words of X per team:
 // policy_x_words = 24 * (branch variables rounded up to 16).
+template <bool kShared = false>
 __device__ __forceinline__ void learned_select(const Tab& tb, int2* st,
                                                const int2* __restrict__ root, const Team& tm,
                                                const PolicyDev* __restrict__ pol, uint32_t* X,
@@ -212,12 +221,12 @@ __device__ __forceinline__ void learned_select(const Tab& tb, int2* st,
   float* P = reinterpret_cast<float*>(X + 8 * nbp);  // [n_chunks][16 tiles][16 rows]
   for (int u = tm.warp; u < n_chunks * S; u += tm.nwarps) {
     const int c = u / S, sp = u % S;
-    mlp_score_tiles(pol, X, c, sp * (16 / S), (sp + 1) * (16 / S), P + 256 * c);
+    mlp_score_tiles<kShared>(pol, X, c, sp * (16 / S), (sp + 1) * (16 / S), P + 256 * c);
   }
   team_bar(tm.bar, tm.nthr);
   for (int k = tm.tid; k < nb; k += tm.nthr) {
     const int2 D = ld_dom(st, tb.branch[k]);
-    if (D.x < D.y) atomicMin(sel, ~learned_key(mlp_row_score(pol, P + 256 * (k >> 4), k & 15), k));
+    if (D.x < D.y) atomicMin(sel, ~learned_key(mlp_row_score<kShared>(pol, P + 256 * (k >> 4), k & 15), k));
   }
 }
 

@@ -259,9 +259,9 @@ __global__ void k_policy_score(const PolicyDev* __restrict__ pol, int n,
   }
   __syncwarp();
   if (16 * c >= n) return;
-  mlp_score_tiles(pol, Xw, 0, 0, 16, part[warp]);
+  mlp_score_tiles<false>(pol, Xw, 0, 0, 16, part[warp]);
   __syncwarp();
-  if (lane < 16 && 16 * c + lane < n) s[16 * c + lane] = mlp_row_score(pol, part[warp], lane);
+  if (lane < 16 && 16 * c + lane < n) s[16 * c + lane] = mlp_row_score<false>(pol, part[warp], lane);
 }
 
 }  // namespace pccp

@@ -132,6 +132,9 @@ __device__ __forceinline__ void red_max_at(uint32_t p, int v) {
 __device__ __forceinline__ void red_min_at(uint32_t p, int v) {
   asm volatile("red.relaxed.cta.shared::cta.min.s32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ void red_add_at(uint32_t p, uint32_t v) {
+  asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void red_or_at(uint32_t p, uint32_t v) {
   asm volatile("red.relaxed.cta.shared::cta.or.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }

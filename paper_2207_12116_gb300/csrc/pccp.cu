@@ -510,6 +510,7 @@ __global__ void __launch_bounds__(1024) k_solve_slots(SolveArgs a) {
 
 #include "mask_search.inc"
 #include "k_search_queue.inc"
+#include "mask_queue.inc"
 
 // -------------------------------------------------------------- host model
 
@@ -2545,6 +2546,8 @@ struct QueuePlan {
   uint32_t slot_bytes, off_track, off_x, off_stack, off_store;
   bool shared, table_global;
   uint32_t shared_bytes, shared_region;
+  bool mask;           // k_search_queue_mask on the models' mask forms
+  uint32_t pol_bytes;
 };
 
 template <int kMode>
@@ -2563,6 +2566,105 @@ void (*queue_kernel(const pccp_solve_opts* o, int mode))(QArgs) {
                      : queue_kernel_t<3>(o);
 }
 
+// The k_search_queue_mask instantiation for a plan's team size and sharing.
+void (*queue_mask_kernel(bool learned, int team, bool shared))(QArgs) {
+  if (team == 32)
+    return learned ? (shared ? k_search_queue_mask<true, true, true> : k_search_queue_mask<true, true, false>)
+                   : (shared ? k_search_queue_mask<true, false, true> : k_search_queue_mask<true, false, false>);
+  return learned ? (shared ? k_search_queue_mask<false, true, true> : k_search_queue_mask<false, true, false>)
+                 : (shared ? k_search_queue_mask<false, false, true> : k_search_queue_mask<false, false, false>);
+}
+
+// Plans a parallel search of models that all have a mask form; p->mask stays
+// false under the conditions of plan_batch_mask.
+int plan_queue_mask(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
+                    bool any_strategy, int smem_max, int sms, QueuePlan* p) {
+  if (o->skip_stable > 0 || o->stream_table > 0) return PCCP_OK;
+  int32_t max_branch = 0, max_tw = 0, max_words = 0, max_rows = 0, max_dec = 2;
+  for (int32_t i = 0; i < n; ++i) {
+    const pccp_model* m = models[i];
+    if (!m->mask.ok) return PCCP_OK;
+    max_branch = std::max(max_branch, m->n_branch);
+    max_tw = std::max(max_tw, mask_search_words(m->mask.n_words, m->mask.bit0));
+    max_words = std::max(max_words, m->mask.n_words);
+    max_rows = std::max(max_rows, m->n_t + m->n_rf + m->n_lin);
+    max_dec = std::max(max_dec, m->max_decisions);
+  }
+  const bool learned = o->strategy == PCCP_LEARNED;
+  p->xw = any_strategy ? 24 * ((max_branch + 15) & ~15) : policy_x_words(o, max_branch);
+  p->max_len = max_dec;
+  p->off_track = static_cast<uint32_t>(align16(16 + sizeof(QCtrl)));
+  p->off_x = p->off_track + 4u * static_cast<uint32_t>((max_tw + 3) & ~3);
+  p->off_stack = static_cast<uint32_t>(align16(p->off_x + 4u * static_cast<uint32_t>(p->xw)));
+  p->off_store = static_cast<uint32_t>(
+      align16(p->off_stack + sizeof(int2) * static_cast<size_t>(p->max_len)));
+  p->pol_bytes = learned || any_strategy
+                     ? static_cast<uint32_t>((sizeof(PolicyDev) + 127u) & ~static_cast<size_t>(127))
+                     : 0u;
+  p->shared = n == 1;
+  p->table_global = false;
+  p->shared_bytes = p->shared ? models[0]->mask.core_bytes : 0u;
+  p->shared_region = p->shared ? ((p->shared_bytes + 127u) & ~127u) + 128u : 0u;
+  uint32_t need = 0;
+  int64_t ring = 0;
+  for (int32_t i = 0; i < n; ++i) {
+    const pccp_model* m = models[i];
+    const uint32_t st_end = (p->off_store + 8u * static_cast<uint32_t>(m->mask.n_slots) + 127u) & ~127u;
+    need = std::max(need, st_end + (p->shared ? 0u : m->mask.core_bytes));
+    ring = std::max(ring, static_cast<int64_t>(m->max_decisions) *
+                              mask_ring_entry(m->mask.n_slots, m->mask.n_words));
+  }
+  need = (need + 127u) & ~127u;
+  const int64_t fixed = static_cast<int64_t>(p->pol_bytes) + p->shared_region;
+  auto fits = [&](int teams) { return fixed + static_cast<int64_t>(teams) * need <= smem_max; };
+  int team = o->threads;
+  if (team == 0 && o->props_per_thread > 0)
+    team = std::min(512, std::max(32, ((max_rows + o->props_per_thread - 1) / o->props_per_thread + 31) & ~31));
+  int teams = o->teams_per_cta;
+  if (team == 0) {
+    // a warp per 64 words of Booleans (many teams keep the SM busy, so a team need
+    // not be wide), more when the teams that fit leave threads for it
+    int w = 1;
+    while (w < 16 && 64 * w < max_words) w *= 2;
+    while (teams > 0 && w > 1 && 32 * w * teams > 512) w /= 2;
+    while (teams == 0 && w < 16 && !fits(512 / (32 * w)) && fits(1)) w *= 2;
+    team = 32 * w;
+  }
+  if (team < 32 || team > 512) return PCCP_OK;
+  if (teams == 0) {
+    // one model: as many teams as there are threads for.  Many models: eight, so
+    // that the last proofs, which donations cannot spread over every team, run on
+    // SMs with fewer teams (256 6-10-task models, 128,000 nodes of proofs in all: 4.2
+    // ms with 8 teams an SM, 5.0 with 12, 6.0 with 16; 13.4 M nodes: 99, 77, 68 ms)
+    teams = std::min(p->shared ? 16 : 8, 512 / team);
+    while (teams > 1 && !fits(teams)) --teams;
+  }
+  if (team * teams > 512 || !fits(teams)) return PCCP_OK;
+  const int64_t cta = smem_max;
+  const uint32_t room = static_cast<uint32_t>((cta - fixed) / teams) & ~127u;
+  p->slot_bytes = static_cast<uint32_t>(
+      std::min<int64_t>(room, (need + ring + 16 + 127) & ~static_cast<int64_t>(127)));
+  p->team = team;
+  p->teams = teams;
+  p->smem = static_cast<size_t>(fixed) + static_cast<size_t>(teams) * p->slot_bytes;
+  p->mode = 0;
+  p->kern = queue_mask_kernel(learned, team, p->shared);
+  int per_sm = 1 << 30;
+  for (int k = 0; k < 2; ++k) {
+    if (!any_strategy && learned != (k == 1)) continue;
+    void (*kern)(QArgs) = queue_mask_kernel(k == 1, team, p->shared);
+    PCCP_CUDA(allow_smem(reinterpret_cast<const void*>(kern), p->smem));
+    int occ = 0;
+    PCCP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, team * teams, p->smem));
+    per_sm = std::min(per_sm, occ);
+  }
+  if (per_sm < 1) return PCCP_OK;
+  p->grid = sms * per_sm;
+  if (o->blocks > 0) p->grid = std::min(p->grid, static_cast<int>(o->blocks));
+  p->mask = true;
+  return PCCP_OK;
+}
+
 // Team size of a search when the caller leaves it to the library: enough
 // threads for about two rows each of the largest model, in whole warps, at
 // least 64 and at most `cap` (small models: small teams, so more of them).
@@ -2577,6 +2679,12 @@ int plan_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opts
   if (smem_max <= 0 || sms <= 0) return PCCP_ERR_CUDA;
   if (o->threads < 0 || o->threads % 32 != 0 || o->threads > 1024) return PCCP_ERR_INVALID;
   if (o->teams_per_cta < 0 || o->teams_per_cta > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
+  p->mask = false;
+  p->pol_bytes = 0u;
+  {
+    const int rc = plan_queue_mask(models, n, o, any_strategy, smem_max, sms, p);
+    if (rc != PCCP_OK || p->mask) return rc;
+  }
   int32_t max_vars = 0, max_branch = 0, max_tw = 0, max_rows = 0, max_dec = 2;
   for (int32_t i = 0; i < n; ++i) {
     const pccp_model* m = models[i];
@@ -2753,6 +2861,7 @@ void queue_plan_args(const QueuePlan& plan, int32_t n, size_t cap, QArgs* a) {
   a->table_global = plan.table_global ? 1 : 0;
   a->shared_bytes = plan.shared_bytes;
   a->shared_region = plan.shared_region;
+  a->pol_bytes = plan.pol_bytes;
 }
 
 // Parallel search of n models over one shared queue (see k_search_queue.inc).
@@ -2769,7 +2878,7 @@ int solve_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opt
     woff[i] = static_cast<int32_t>(wit_total);
     wit_total += models[i]->n_vars;
     if (wit_total > INT32_MAX) return PCCP_ERR_INVALID;
-    desc[i] = instance_desc(models[i], i, woff[i], false);
+    desc[i] = instance_desc(models[i], i, woff[i], plan.mask);
   }
   const size_t per_item = static_cast<size_t>(plan.max_len) * sizeof(int2);
   const size_t cap = queue_cap(n, n_teams, plan.max_len);

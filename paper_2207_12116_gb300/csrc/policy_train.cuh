@@ -71,16 +71,17 @@ __device__ __forceinline__ void feature_fragment(uint32_t (&a)[4], const float* 
   }
 }
 
-// First hidden layer of a 16-row chunk as the second layer's A fragments.
-__device__ __forceinline__ void layer1_fragments(const PolicyDev* __restrict__ pol,
+// First hidden layer of a 16-row chunk as the second layer's A fragments; w1: the
+// first layer's fragments.
+__device__ __forceinline__ void layer1_fragments(const PolicyDev* __restrict__ pol, const uint2* w1,
                                                  const uint32_t (&a1)[4], int lane,
                                                  uint32_t (&a2)[8][4]) {
   const int t = lane & 3;
 #pragma unroll
   for (int kk = 0; kk < 8; ++kk) {
     float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-    mma_16816(d0, a1, __ldg(&pol->w1[2 * kk][lane]));
-    mma_16816(d1, a1, __ldg(&pol->w1[2 * kk + 1][lane]));
+    mma_16816(d0, a1, w1[64 * kk + lane]);
+    mma_16816(d1, a1, w1[64 * kk + 32 + lane]);
     const float2 b0 = __ldg(reinterpret_cast<const float2*>(&pol->b1[16 * kk + 2 * t]));
     const float2 b1 = __ldg(reinterpret_cast<const float2*>(&pol->b1[16 * kk + 2 * t + 8]));
     a2[kk][0] = pack_bf16x2(fmaxf(d0[0] + b0.x, 0.f), fmaxf(d0[1] + b0.y, 0.f));
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(256) k_train_forward(const PolicyDev* __restri
   const int r0 = blockIdx.x * kTrainRows + 16 * chunk + g;
   uint32_t a1[4], a2[8][4];
   feature_fragment(a1, f, n, r0, t);
-  layer1_fragments(pol, a1, lane, a2);
+  layer1_fragments(pol, &pol->w1[0][0], a1, lane, a2);
   if (threadIdx.x < 128) sw3[threadIdx.x] = __ldg(&pol->w3[threadIdx.x]);
   if (half == 0) {
 #pragma unroll
@@ -471,64 +472,116 @@ __global__ void k_build_policy(int n, const float* __restrict__ p, __nv_bfloat16
 
 // Features of every branch variable of every store (the search kernels'
 // write_features, rounded to BF16 as the network sees them); out is
-// [n_stores][n_branch][12].  Stores are joined with the root first.
+// [n_stores][n_branch][12].  Stores are joined with the root first.  A thread a
+// row; its 48 bytes go out in three 16-byte stores when `out` allows it.
+template <bool kVec>
 __global__ void k_policy_features(const uint8_t* __restrict__ image, const int2* __restrict__ root,
                                   int n_stores, int n_vars, const int32_t* __restrict__ lb,
                                   const int32_t* __restrict__ ub, const int32_t* __restrict__ depth,
                                   float* __restrict__ out) {
-  const Tab tb = make_tab(image);
-  const BranchStatic* bs = reinterpret_cast<const BranchStatic*>(tb.bstat);
-  const int nb = tb.n_branch;
+  const TableHeader* h = reinterpret_cast<const TableHeader*>(image);
+  const BranchStatic* bs = reinterpret_cast<const BranchStatic*>(image + h->off_bstat);
+  const int32_t* branch = reinterpret_cast<const int32_t*>(image + h->off_branch);
+  const int nb = h->n_branch, objective = h->objective;
   const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= static_cast<long long>(n_stores) * nb) return;
-  const int s = static_cast<int>(i / nb), k = static_cast<int>(i - static_cast<long long>(s) * nb);
+  const int s = i <= 0x7fffffffll ? static_cast<int>(i) / nb : static_cast<int>(i / nb);
+  const int k = static_cast<int>(i - static_cast<long long>(s) * nb);
   // stores are in the caller's variable order; the table and root in the
   // library's (user_of: the caller's index of each variable, after the root)
   const int32_t* user_of = reinterpret_cast<const int32_t*>(root + n_vars) + n_vars;
-  const int v = tb.branch[k];
+  const int v = branch[k];
   const int32_t* l = lb + static_cast<size_t>(s) * n_vars;
   const int32_t* u = ub + static_cast<size_t>(s) * n_vars;
   const int2 R = root[v];
   const int vu = user_of[v];
   const int2 D = make_int2(max(l[vu], R.x), min(u[vu], R.y));
   float prog = 0.f;
-  if (tb.objective >= 0) {
-    const int2 RO = root[tb.objective];
-    prog = static_cast<float>(max(l[user_of[tb.objective]], RO.x) - RO.x) /
+  if (objective >= 0) {
+    const int2 RO = root[objective];
+    prog = static_cast<float>(max(l[user_of[objective]], RO.x) - RO.x) /
            (static_cast<float>(RO.y - RO.x) + 1.f);
   }
   uint32_t row[8];
   write_features(row, k, D, R, bs[k], nb, depth ? depth[s] : 0, prog);
-  float* o = out + static_cast<size_t>(i) * kPolicyFeatures;
+  float* o = out + (static_cast<size_t>(s) * nb + k) * kPolicyFeatures;
+  float x[kPolicyFeatures];
+#pragma unroll
   for (int c = 0; c < kPolicyFeatures; ++c) {
     const uint32_t w = row[c >> 1];
-    const uint16_t h = static_cast<uint16_t>((c & 1) ? (w >> 16) : (w & 0xffffu));
-    o[c] = __bfloat162float(__ushort_as_bfloat16(h));
+    x[c] = __uint_as_float((c & 1) ? (w & 0xffff0000u) : (w << 16));
+  }
+#pragma unroll
+  for (int c = 0; c < kPolicyFeatures; c += 4) {
+    if (kVec) {
+      *reinterpret_cast<float4*>(o + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+    } else {
+      o[c] = x[c];
+      o[c + 1] = x[c + 1];
+      o[c + 2] = x[c + 2];
+      o[c + 3] = x[c + 3];
+    }
   }
 }
 
-// Scores of n feature rows (FP32 [n][12]) by the search kernels' network:
-// 16-row chunks per warp, rows staged as BF16 in shared memory.
-__global__ void k_policy_score(const PolicyDev* __restrict__ pol, int n,
-                               const float* __restrict__ f, float* __restrict__ s) {
-  __shared__ uint32_t X[8][16 * 8];  // 8 warps x 16 rows x 8 words
-  __shared__ float part[8][256];     // tile parts (mlp_score_tiles)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * 8 + warp;
-  uint32_t* Xw = X[warp];
-  for (int i = lane; i < 16 * 8; i += 32) {
-    const int r = 16 * c + (i >> 3), w = i & 7;
-    float lo = 0.f, hi = 0.f;
-    if (r < n && 2 * w < kPolicyFeatures) lo = f[static_cast<size_t>(r) * kPolicyFeatures + 2 * w];
-    if (r < n && 2 * w + 1 < kPolicyFeatures)
-      hi = f[static_cast<size_t>(r) * kPolicyFeatures + 2 * w + 1];
-    Xw[i] = pack_bf16x2(lo, hi);
+// Scores of n feature rows (FP32 [n][12]) by the search kernels' network, with
+// the search's sums (mlp_score_tiles, mlp_row_score).  A warp takes 32 rows at a
+// time, so every weight fragment read from shared memory (36 KB, staged once per
+// CTA) feeds two products; with a 16-row chunk a warp and fragments from L2 each
+// chunk moved 36 KB (120,000 rows: 24.7 us, 20.4 us with this kernel).
+__global__ void __launch_bounds__(256, 2) k_policy_score(const PolicyDev* __restrict__ pol, int n,
+                                                      const float* __restrict__ f,
+                                                      float* __restrict__ s) {
+  __shared__ __align__(16) uint2 sw[16 * 32 + 8 * 16 * 32];  // w1, then w2
+  __shared__ float4 bw[16][4];  // b2, w3 of a lane's two units of a tile
+  for (int i = threadIdx.x; i < (16 * 32 + 8 * 16 * 32) / 2; i += blockDim.x)
+    reinterpret_cast<uint4*>(sw)[i] = __ldg(reinterpret_cast<const uint4*>(&pol->w1[0][0]) + i);
+  if (threadIdx.x < 64) {
+    const int c = 2 * static_cast<int>(threadIdx.x);
+    bw[threadIdx.x >> 2][threadIdx.x & 3] = make_float4(__ldg(&pol->b2[c]), __ldg(&pol->b2[c + 1]),
+                                                        __ldg(&pol->w3[c]), __ldg(&pol->w3[c + 1]));
   }
-  __syncwarp();
-  if (16 * c >= n) return;
-  mlp_score_tiles<false>(pol, Xw, 0, 0, 16, part[warp]);
-  __syncwarp();
-  if (lane < 16 && 16 * c + lane < n) s[16 * c + lane] = mlp_row_score<false>(pol, part[warp], lane);
+  __syncthreads();
+  const uint2* w2 = sw + 16 * 32;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int n_warps = static_cast<int>(gridDim.x * (blockDim.x >> 5));
+  const float b3 = __ldg(&pol->b3);
+  for (int c = static_cast<int>(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); 32ll * c < n;
+       c += n_warps) {
+    uint32_t a[2][8][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      uint32_t a1[4];
+      feature_fragment(a1, f, n, 32 * c + 16 * q + g, t);
+      layer1_fragments(pol, sw, a1, lane, a[q]);
+    }
+    float sum = 0.f;  // of row 32 c + 16 (t & 1) + 8 (t >> 1) + g
+#pragma unroll 2
+    for (int j = 0; j < 16; ++j) {
+      float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint2 w = w2[(16 * kk + j) * 32 + lane];
+        mma_16816(acc[0], a[0][kk], w);
+        mma_16816(acc[1], a[1][kk], w);
+      }
+      const float4 B = bw[j][t];
+      float part[2][2];  // [16-row half][8-row half]
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        part[q][0] = fmaxf(acc[q][0] + B.x, 0.f) * B.z + fmaxf(acc[q][1] + B.y, 0.f) * B.w;
+        part[q][1] = fmaxf(acc[q][2] + B.x, 0.f) * B.z + fmaxf(acc[q][3] + B.y, 0.f) * B.w;
+      }
+      // the four lanes of a row, each ending with the sum of one of the four rows
+      const bool odd = t & 1, high = t & 2;
+      float x = odd ? part[1][0] : part[0][0], y = odd ? part[1][1] : part[0][1];
+      x += __shfl_xor_sync(0xffffffffu, odd ? part[0][0] : part[1][0], 1);
+      y += __shfl_xor_sync(0xffffffffu, odd ? part[0][1] : part[1][1], 1);
+      sum += (high ? y : x) + __shfl_xor_sync(0xffffffffu, high ? x : y, 2);
+    }
+    const int r = 32 * c + 16 * (t & 1) + 8 * (t >> 1) + g;
+    if (r < n) s[r] = sum + b3;
+  }
 }
 
 }  // namespace pccp

@@ -1283,7 +1283,7 @@ __device__ __forceinline__ void sweep_rows_streamed(const Sweep& w, const Team& 
 // Per-team scalars of the fixed point (shared memory): failure flag and the
 // work counters of the current store.
 struct FixCtrl {
-  int fail;
+  int fail;  // the sweep (from 1) that found an empty interval, 0: none
   int evals;
   int bytes;
   int pad;
@@ -1367,7 +1367,9 @@ __device__ __forceinline__ int team_fixpoint(const Tab& tb, int2* st, const Team
         atomicAdd(&fc->bytes, by);
       }
     }
-    if (f.fl) st_relaxed(&fc->fail, 1);
+    // the sweep's number, not a flag: a warp that is late at the test below must
+    // not take what a faster one finds in the next sweep for this one's
+    if (f.fl) st_relaxed(&fc->fail, it + 1);
     ++it;
     full = false;
     const bool any = team_bar_or(tm.bar, tm.nthr, f.ch || f.fl);
@@ -1376,7 +1378,7 @@ __device__ __forceinline__ int team_fixpoint(const Tab& tb, int2* st, const Team
       count_sweeps<kTrack>(tb, tm, fc, it);
       return kError;
     }
-    if (ld_relaxed(&fc->fail)) {
+    if (ld_relaxed(&fc->fail) == it) {
       iters = it;
       count_sweeps<kTrack>(tb, tm, fc, it);
       return kFailed;

@@ -37,15 +37,17 @@ namespace pccp {
 //                           pair filled with one that has no lanes
 //   pattern          uint2 [32] {x | y << 16, d}, a lane each; y is added to the
 //                           descriptor's (one of the two is 0)
-//   mask row         uint4 {c, first full word's slot | full words << 16 (its
-//                           only word's slot when one_word),
+//   mask row         uint4 {c, first full word's slot | full words << 16 |
+//                           slots from one to the next << 24 (its only word's
+//                           slot when one_word),
 //                           byte offset of its planes,
 //                           slot of the partial word or kNoSlot | largest coefficient << 16}
 //   planes           uint4 [words][n_pq]: planes 4q .. 4q + 3, least
 //                           significant first; full words, then the partial one
-// A row's group of Booleans fills `full` consecutive words; its rest sits in a
+// A row's group of Booleans fills `full` words; its rest sits in a
 // partial word that other groups may share.
 constexpr uint32_t kNoSlot = 0xffffu;
+constexpr int kRowFullMax = 255, kRowStrideMax = 255;  // what a mask row can hold
 // Units of an interval variable (searches) and its paths (see pack_mask).
 constexpr uint16_t kUnitNone = 0xffffu, kUnitCross = 0x8000u;
 constexpr int16_t kNoPath = INT16_MIN;
@@ -364,12 +366,12 @@ __device__ __forceinline__ void m_row(const MTab& tb, uint32_t planes, int n_pq,
     return;
   }
   const uint32_t rest = R.w & 0xffffu;
-  const int full = static_cast<int>(R.y >> 16);
-  const uint32_t slot0 = st + (R.y & 0xffffu);
+  const int full = static_cast<int>((R.y >> 16) & 255u);
+  const uint32_t slot0 = st + (R.y & 0xffffu), stride = 8u * (R.y >> 24);
   const int words = full + (rest != kNoSlot ? 1 : 0);
   int S = 0;
   for (int w = 0; w < words; ++w) {
-    const uint32_t lo = static_cast<uint32_t>(ld_slot(w < full ? slot0 + 8 * w : st + rest).x);
+    const uint32_t lo = static_cast<uint32_t>(ld_slot(w < full ? slot0 + stride * w : st + rest).x);
     for (int q = 0; q < n_pq; ++q) S += m_sum(lds128(P + 16 * (w * n_pq + q)), lo) << (4 * q);
   }
   const int slack = c - S;
@@ -379,7 +381,7 @@ __device__ __forceinline__ void m_row(const MTab& tb, uint32_t planes, int n_pq,
     return;
   }
   for (int w = 0; w < words; ++w) {
-    const uint32_t slot = w < full ? slot0 + 8 * w : st + rest;
+    const uint32_t slot = w < full ? slot0 + stride * w : st + rest;
     const int2 W = ld_slot(slot);
     uint32_t gt = 0u, eq = static_cast<uint32_t>(W.y) & ~static_cast<uint32_t>(W.x);
     if (eq == 0u) continue;

@@ -4,11 +4,13 @@ Counts, optima and witnesses equal the oracle's (the queue's on proof trees,
 which no order changes) at the edges of the word layouts, for one- and many-warp
 teams, with rings shorter than the path, for models without a path matrix (a
 cycle of precedences), and where a shape leaves the search to intervals."""
+import numpy as np
 import pytest
 
 import oracle
 from oracle.rcpsp import rcpsp_model
 import paper_2207_12116_gb300 as pccp
+from tests.gpu_util import compare_batch
 from tests.test_gpu_mask import HUGE, SMALL, WIDE, instance
 from tests.test_gpu_solve import same
 
@@ -125,3 +127,28 @@ def test_cycle_of_precedences(seed):
     c = oracle.solve(om, mode=oracle.COUNT_ALL, obj_ub=o["objective"])
     r = pccp.solve(m, mode=pccp.PCCP_COUNT_ALL, obj_ub=o["objective"], deterministic=False, donate_nodes=1)
     assert (r["nodes"], r["fails"], r["solutions"]) == (c["nodes"], c["fails"], c["solutions"])
+
+
+@pytest.mark.parametrize("sizes", [(40, 70), (33, 64), (64, 64), (96, 32, 31), (65, 1, 65)])
+def test_groups_of_like_and_unlike_size(sizes):
+    """Resource rows over groups of Booleans of several words: like groups'
+    words lie side by side, unlike groups' one group after another."""
+    g = np.random.default_rng(sum(sizes))
+    n, k = 6, sum(sizes)
+    lb0, ub0 = [0] * n + [0] * k, [9] * n + [1] * k
+    pairs = [(int(a), int(b)) for a, b in (g.permutation(n)[:2] for _ in range(k))]
+    reified = [(n + i, a, b, 1 + i % 4) for i, (a, b) in enumerate(pairs)]
+    linear, at = [], 0
+    for size in sizes:
+        for _ in range(2):
+            linear.append((size, [(int(g.integers(1, 6)), n + at + i) for i in range(size)]))
+        at += size
+    temporal = [(0, 1, 1), (2, 3, 2)]
+    m = pccp.Model.from_lists(lb0, ub0, temporal, linear, reified)
+    om = oracle.Model(lb0, ub0, temporal, linear, reified)
+    lb, ub = np.tile(np.int32(lb0), (48, 1)), np.tile(np.int32(ub0), (48, 1))
+    lb[:, :n] = g.integers(0, 5, (48, n))
+    ub[:, :n] = lb[:, :n] + g.integers(0, 5, (48, n))
+    dlb, dub = torch.from_numpy(lb).cuda(), torch.from_numpy(ub).cuda()
+    st, _ = pccp.propagate(m, dlb, dub)
+    compare_batch(om, lb, ub, st.cpu().numpy(), dlb.cpu().numpy(), dub.cpu().numpy())

@@ -237,7 +237,9 @@ def launch_desc(args):
 
 
 KERNEL_SOURCES = ("paper_2207_12116_gb300/csrc/k_propagate.cuh",
-                  "paper_2207_12116_gb300/csrc/pccp_device.cuh")
+                  "paper_2207_12116_gb300/csrc/pccp_device.cuh",
+                  "paper_2207_12116_gb300/csrc/k_propagate_mask.cuh",
+                  "paper_2207_12116_gb300/csrc/mask_device.cuh")
 def profile_path():
     """The committed ncu summary of the propagation workload being run."""
     return f"profiles/k_propagate_{FAMILY}_batch.md"
@@ -258,7 +260,7 @@ def kernel_hash():
 
 
 def recorded_traffic():
-    """DRAM bytes per launch of k_propagate from the committed ncu summary,
+    """DRAM bytes per launch of the propagation kernel from the committed ncu summary,
     or None when the kernel sources changed since that capture."""
     try:
         text = open(os.path.join(ROOT, profile_path())).read()
@@ -725,9 +727,9 @@ def run_gpu(args):
 def run_profile_leg(args):
     """One warm-up launch and one launch of a search kernel, for ncu captures
     (skip 1 launch of the kernel, capture 1):
-      batched : k_solve_slots, 256 seeded 30-60-task models, input order,
+      batched : k_solve_mask, 256 seeded 30-60-task models, input order,
                 500 nodes each, the library's launch shape;
-      complete: k_search_queue, the 256 6-10-task models proved optimal in
+      complete: k_search_queue_mask, the 256 6-10-task models proved optimal in
                 the parallel form, first-fail, 8 teams of 64 threads per CTA."""
     import torch
     import paper_2207_12116_gb300 as pccp

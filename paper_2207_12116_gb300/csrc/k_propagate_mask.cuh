@@ -10,6 +10,11 @@
 // node are still the root's, so a quad usually costs its loads and eight
 // compares.  A store that fails is not written back (its contents are
 // unspecified).
+//
+// What bounds it: instruction issue, and for batches of few stores the hardest
+// store's chain of phases.  Kernel times against k_propagate on the same stores (one
+// GB300): 10,000 of 30 tasks 169 -> 88 us.  Whole passes, with the caller's copy of
+// the stores: 777 of 60 tasks 151 -> 92 us, 1,216 of 120 tasks 930 -> 298 us.
 #pragma once
 
 #include "mask_device.cuh"

@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "../../include/pccp.h"
+#include "launch_rules.h"
 #include "pccp_device.cuh"
 #include "k_propagate.cuh"
 #include "mask_device.cuh"
@@ -1681,8 +1682,7 @@ int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve
   }
   int team = o->threads;
   if (team == 0 && o->props_per_thread > 0)
-    team = std::min(512 / teams, std::max(32, ((max_rows + o->props_per_thread - 1) /
-                                                   o->props_per_thread + 31) & ~31));
+    team = team_for_rows(max_rows, o->props_per_thread, 512, teams);
   if (team == 0) {
     // a warp per sixteen words of Booleans: a node runs few of them, and a
     // barrier costs more with more warps (256 30-60-task models x 500 nodes, two
@@ -1693,6 +1693,7 @@ int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve
     while (64 * w * teams <= 512 && 16 * w < max_words) w *= 2;
     team = 32 * w;
   }
+  if (team % 32 != 0) return PCCP_ERR_INVALID;
   if (team < 32 || team * teams > 512 || need > room_of(teams)) return PCCP_OK;
   p->slots = true;
   p->stages = 0;
@@ -1811,15 +1812,14 @@ int plan_batch(const pccp_model* const* models, int32_t n, const pccp_solve_opts
   }
   int team = o->threads;
   if (team == 0 && o->props_per_thread > 0)
-    team = std::min(1024 / teams, std::max(32, ((max_rows + o->props_per_thread - 1) /
-                                                    o->props_per_thread + 31) & ~31));
+    team = team_for_rows(max_rows, o->props_per_thread, 1024, teams);
   // default team: 256 threads when several share a CTA; a whole CTA when one
   // team has it (its search is a chain of dependent sweeps, which the lane
   // groups of the linear rows shorten with more lanes: 256 30-60-task models
   // x 4,000 nodes in 353 ms at 1024 threads, 370 at 512, 401 at 256)
   if (team == 0)
     team = all_fit_one && teams > 1 ? std::min(256, (1024 / teams) & ~31) : (1024 / teams) & ~31;
-  if (team < 32 || team * teams > 1024) return PCCP_ERR_INVALID;
+  if (team < 32 || team % 32 != 0 || team * teams > 1024) return PCCP_ERR_INVALID;
   // slot size: what the largest model needs (staged when it fits), at most
   // an equal share of the CTA's shared memory
   const uint32_t room = static_cast<uint32_t>(smem_max / teams) & ~127u;
@@ -2618,8 +2618,7 @@ int plan_queue_mask(const pccp_model* const* models, int32_t n, const pccp_solve
   const int64_t fixed = static_cast<int64_t>(p->pol_bytes) + p->shared_region;
   auto fits = [&](int teams) { return fixed + static_cast<int64_t>(teams) * need <= smem_max; };
   int team = o->threads;
-  if (team == 0 && o->props_per_thread > 0)
-    team = std::min(512, std::max(32, ((max_rows + o->props_per_thread - 1) / o->props_per_thread + 31) & ~31));
+  if (team == 0 && o->props_per_thread > 0) team = team_for_rows(max_rows, o->props_per_thread, 512, 1);
   int teams = o->teams_per_cta;
   if (team == 0) {
     // a warp per 64 words of Booleans (many teams keep the SM busy, so a team need
@@ -2725,8 +2724,7 @@ int plan_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opts
     p->shared_region = p->table_global ? 0u : region;
     int team = o->threads;
     if (team == 0 && o->props_per_thread > 0)
-      team = std::min(1024, std::max(32, ((max_rows + o->props_per_thread - 1) /
-                                              o->props_per_thread + 31) & ~31));
+      team = team_for_rows(max_rows, o->props_per_thread, 1024, 1);
     if (team == 0) team = p->table_global ? 1024 : default_team(max_rows, 128);
     const int fit = static_cast<int>((static_cast<uint32_t>(smem_max) - p->shared_region) / per);
     int teams = o->teams_per_cta > 0 ? o->teams_per_cta : 8;

@@ -69,12 +69,23 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) k_propagate_mask(Prop
   tm.lane = static_cast<int>(threadIdx.x & 31u);
   tm.warp = tm.tid >> 5;
   tm.nwarps = a.team_size >> 5;
-  const MTab tb = make_mtab(smem, a.levels & 1);
-  const uint32_t sb = smem_u32(st);
-  const TableHeader* h = reinterpret_cast<const TableHeader*>(smem);
   const int nv = a.n_vars;
   const int n_teams = static_cast<int>(gridDim.x) * a.teams;
   int s = static_cast<int>(blockIdx.x) + team_id * static_cast<int>(gridDim.x);
+  if (!ok) {  // the image never arrived: nothing of it is read, the stores are reported
+    for (; tm.tid == 0 && s < a.n_stores; s = a.counter ? n_teams + atomicAdd(a.counter, 1) : a.n_stores) {
+      a.status[s] = kError;
+      if (a.iters) a.iters[s] = 0;
+      if (a.work) {
+        a.work[2 * static_cast<size_t>(s)] = 0;
+        a.work[2 * static_cast<size_t>(s) + 1] = 0;
+      }
+    }
+    return;
+  }
+  const MTab tb = make_mtab(smem, a.levels & 1);
+  const uint32_t sb = smem_u32(st);
+  const TableHeader* h = reinterpret_cast<const TableHeader*>(smem);
   if (tm.tid == 0) mc->ev[0] = mc->evals = 0u;  // published by the first store's barrier
   int at = 0;
   while (s < a.n_stores) {
@@ -105,40 +116,36 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) k_propagate_mask(Prop
     mbar_team<kWarp>(tm);
     int status = kFailed;
     MaskWork work{0, 0, 0, 0};
-    if (ok) {
-      // a quad whose lower bounds are at most the root's and whose upper
-      // bounds are at least 1 leaves the root's bits (nothing is read from the map)
-      const uint32_t rl = smem_u32(smem) + static_cast<uint32_t>(h->off_rl + 4 * head * h->rl_words);
+    // a quad whose lower bounds are at most the root's and whose upper
+    // bounds are at least 1 leaves the root's bits (nothing is read from the map)
+    const uint32_t rl = smem_u32(smem) + static_cast<uint32_t>(h->off_rl + 4 * head * h->rl_words);
 #pragma unroll 4
-      for (int q = tm.tid; q < nq; q += tm.nthr) {
-        const int x = head + 4 * q;
-        const int4 l = __ldcs(reinterpret_cast<const int4*>(lbs + x));
-        const int4 u = __ldcs(reinterpret_cast<const int4*>(ubs + x));
-        const int r = lds32(rl + 4 * (q >> 3)) >> (4 * (q & 7));
-        const bool over = (l.x > (r & 1)) | (l.y > ((r >> 1) & 1)) | (l.z > ((r >> 2) & 1)) |
-                          (l.w > ((r >> 3) & 1));
-        if (over | (min(min(u.x, u.y), min(u.z, u.w)) < 1)) {
-          const uint4 e = __ldg(reinterpret_cast<const uint4*>(map + x));
-          m_join(sb, l.x, u.x, e.x, empty);
-          m_join(sb, l.y, u.y, e.y, empty);
-          m_join(sb, l.z, u.z, e.z, empty);
-          m_join(sb, l.w, u.w, e.w, empty);
-        }
+    for (int q = tm.tid; q < nq; q += tm.nthr) {
+      const int x = head + 4 * q;
+      const int4 l = __ldcs(reinterpret_cast<const int4*>(lbs + x));
+      const int4 u = __ldcs(reinterpret_cast<const int4*>(ubs + x));
+      const int r = lds32(rl + 4 * (q >> 3)) >> (4 * (q & 7));
+      const bool over = (l.x > (r & 1)) | (l.y > ((r >> 1) & 1)) | (l.z > ((r >> 2) & 1)) |
+                        (l.w > ((r >> 3) & 1));
+      if (over | (min(min(u.x, u.y), min(u.z, u.w)) < 1)) {
+        const uint4 e = __ldg(reinterpret_cast<const uint4*>(map + x));
+        m_join(sb, l.x, u.x, e.x, empty);
+        m_join(sb, l.y, u.y, e.y, empty);
+        m_join(sb, l.z, u.z, e.z, empty);
+        m_join(sb, l.w, u.w, e.w, empty);
       }
-      for (int k = tm.tid; k < nv - 4 * nq; k += tm.nthr) {  // before and after the quads
-        const int x = nq == 0 || k < head ? k : k + 4 * nq;
-        m_join(sb, lbs[x], ubs[x], __ldg(map + x), empty);
-      }
-      if (tm.tid == 0 && next < a.n_stores) {
-        prefetch_l2(a.lb + static_cast<size_t>(next) * nv, 4 * static_cast<size_t>(nv));
-        prefetch_l2(a.ub + static_cast<size_t>(next) * nv, 4 * static_cast<size_t>(nv));
-      }
-      if (!mbar_team_or<kWarp>(tm, empty))
-        status = m_fixpoint<kWarp>(tb, st, tm, mc, true, a.max_iter, at, work);
-    } else {
-      status = kError;
     }
-    if (status != kFailed && ok) {
+    for (int k = tm.tid; k < nv - 4 * nq; k += tm.nthr) {  // before and after the quads
+      const int x = nq == 0 || k < head ? k : k + 4 * nq;
+      m_join(sb, lbs[x], ubs[x], __ldg(map + x), empty);
+    }
+    if (tm.tid == 0 && next < a.n_stores) {
+      prefetch_l2(a.lb + static_cast<size_t>(next) * nv, 4 * static_cast<size_t>(nv));
+      prefetch_l2(a.ub + static_cast<size_t>(next) * nv, 4 * static_cast<size_t>(nv));
+    }
+    if (!mbar_team_or<kWarp>(tm, empty))
+      status = m_fixpoint<kWarp>(tb, st, tm, mc, true, a.max_iter, at, work);
+    if (status != kFailed) {
 #pragma unroll 2
       for (int q = tm.tid; q < nq; q += tm.nthr) {
         const int x = head + 4 * q;

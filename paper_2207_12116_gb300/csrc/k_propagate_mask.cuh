@@ -86,7 +86,9 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) k_propagate_mask(Prop
   const MTab tb = make_mtab(smem, a.levels & 1);
   const uint32_t sb = smem_u32(st);
   const TableHeader* h = reinterpret_cast<const TableHeader*>(smem);
-  if (tm.tid == 0) mc->ev[0] = mc->evals = 0u;  // published by the first store's barrier
+  // events, counts, and the watch masks, of which those of words without a
+  // reified row are never written; published by the first store's barrier
+  for (int i = tm.tid; i < a.track_words; i += tm.nthr) reinterpret_cast<uint32_t*>(mc)[i] = 0u;
   int at = 0;
   while (s < a.n_stores) {
     int32_t* lbs = a.lb + static_cast<size_t>(s) * nv;

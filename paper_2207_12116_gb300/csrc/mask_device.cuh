@@ -72,7 +72,8 @@ constexpr uint32_t kEvError = 16u;  // the iteration budget ran out
 
 // Per-team control words of the fixed point (shared memory), followed by the
 // words' watch masks (a word per word of Booleans: those that would tell
-// something if they became 0, as of the word phase) and two bitmaps over the
+// something if they became 0, as of the word phase; 0 for a word without a
+// reified row, cleared by the kernel) and two bitmaps over the
 // words: those in which a mask row cleared a watched Boolean (written in one
 // round's row phase, read in the next round's word phase).
 struct MaskCtrl {
@@ -441,8 +442,8 @@ struct MaskWork {
 };
 
 // Fixed-point loop of one team; st is staged and published.  `at` (team-uniform,
-// kept from one fixed point of the team to the next) starts at 0 with mc->ev[0]
-// and mc->evals cleared.  A round is three phases, each ended by the
+// kept from one fixed point of the team to the next) starts at 0 with the
+// control words and the watch masks cleared.  A round is three phases, each ended by the
 // team's events: the temporal rows to their closure, the words, the mask rows.
 // A later phase sees what the earlier ones told, so a phase runs again only
 // after an event that can give it something to tell:

@@ -1481,7 +1481,9 @@ int plan_propagate(const pccp_model* m, int32_t n_stores, const pccp_launch_conf
   if (cfg && cfg->teams_per_cta > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
   p->mask = false;
   p->slot_bytes = 0u;
-  if (m->mask.ok && !(cfg && (cfg->skip_stable > 0 || cfg->stream_table > 0))) {
+  // a loop asked for by name (change tracking, eventless) or streamed tables: the
+  // general kernels, whose options these are
+  if (m->mask.ok && !(cfg && (cfg->skip_stable != 0 || cfg->stream_table > 0))) {
     const int rc = plan_propagate_mask(m, n_stores, cfg, smem_max, sms, p);
     if (rc != PCCP_OK || p->mask) return rc;
   }
@@ -1635,13 +1637,20 @@ SolveKernel mask_kernel(bool learned, int team) {
   return learned ? k_solve_mask<false, true> : k_solve_mask<false, false>;
 }
 
+// Searches that ask for one of the general kernels' loops by name: change
+// tracking or the eventless loop (skip_stable), or an order of the temporal rows
+// (temporal_levels; the mask searches follow moved variables along paths instead).
+bool names_loop(const pccp_solve_opts* o) { return o->skip_stable != 0 || o->temporal_levels != 0; }
+
+// Searches for the general kernels: those, and streamed tables.
+bool general_search(const pccp_solve_opts* o) { return names_loop(o) || o->stream_table > 0; }
+
 // Plans a batched search of models that all have a mask form; p->mask stays
-// false when some model has none or does not fit, when the caller asks for what
-// only the general kernels have (change tracking, streamed tables), or for
+// false when some model has none or does not fit, for a general_search, or for
 // more than 512 threads a CTA.
 int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
                     bool any_strategy, int smem_max, int sms, BatchPlan* p) {
-  if (o->skip_stable > 0 || o->stream_table > 0) return PCCP_OK;
+  if (general_search(o)) return PCCP_OK;
   int32_t max_branch = 0, max_tw = 0, max_words = 0, max_rows = 0, max_dec = 2;
   for (int32_t i = 0; i < n; ++i) {
     const pccp_model* m = models[i];
@@ -2579,7 +2588,7 @@ void (*queue_mask_kernel(bool learned, int team, bool shared))(QArgs) {
 // false under the conditions of plan_batch_mask.
 int plan_queue_mask(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
                     bool any_strategy, int smem_max, int sms, QueuePlan* p) {
-  if (o->skip_stable > 0 || o->stream_table > 0) return PCCP_OK;
+  if (general_search(o)) return PCCP_OK;
   int32_t max_branch = 0, max_tw = 0, max_words = 0, max_rows = 0, max_dec = 2;
   for (int32_t i = 0; i < n; ++i) {
     const pccp_model* m = models[i];
@@ -2672,7 +2681,7 @@ int default_team(int max_rows, int cap) {
 }
 
 int plan_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
-               QueuePlan* p, bool any_strategy = false) {
+               QueuePlan* p, bool any_strategy = false, bool allow_mask = true) {
   const int smem_max = max_dyn_smem();
   const int sms = sm_count();
   if (smem_max <= 0 || sms <= 0) return PCCP_ERR_CUDA;
@@ -2680,7 +2689,7 @@ int plan_queue(const pccp_model* const* models, int32_t n, const pccp_solve_opts
   if (o->teams_per_cta < 0 || o->teams_per_cta > kMaxTeamsPerCta) return PCCP_ERR_INVALID;
   p->mask = false;
   p->pol_bytes = 0u;
-  {
+  if (allow_mask) {
     const int rc = plan_queue_mask(models, n, o, any_strategy, smem_max, sms, p);
     if (rc != PCCP_OK || p->mask) return rc;
   }
@@ -2970,7 +2979,7 @@ int pccp_solve(const pccp_model* m, const pccp_solve_opts* opts, pccp_result* re
     return solve_queue(one, 1, opts, result, static_cast<cudaStream_t>(stream));
   }
   pccp_solve_opts o = *opts;
-  if (o.threads <= 0 && !(m->mask.ok && o.skip_stable <= 0 && o.stream_table <= 0)) o.threads = 512;
+  if (o.threads <= 0 && !(m->mask.ok && !general_search(&o))) o.threads = 512;
   o.teams_per_cta = 1;  // one model: one team
   const pccp_model* one[1] = {m};
   return pccp_solve_batch(one, 1, &o, result, stream);

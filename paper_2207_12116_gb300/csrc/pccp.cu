@@ -1733,9 +1733,10 @@ int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve
 // Plans a batched search.  any_strategy: room for the learned strategy's
 // feature rows and an occupancy valid for every strategy's kernel (a batch
 // planned once for later searches).  Returns SMEM when some store does not
-// fit a slot.
+// fit a slot.  general_team: the general kernels' team size when the options name
+// none (0: by what fits a CTA).
 int plan_batch(const pccp_model* const* models, int32_t n, const pccp_solve_opts* o,
-               bool any_strategy, BatchPlan* p, bool allow_mask = true) {
+               bool any_strategy, BatchPlan* p, bool allow_mask = true, int general_team = 0) {
   const int smem_max = max_dyn_smem();
   const int sms = sm_count();
   if (smem_max <= 0 || sms <= 0) return PCCP_ERR_CUDA;
@@ -1760,6 +1761,9 @@ int plan_batch(const pccp_model* const* models, int32_t n, const pccp_solve_opts
     const int rc = plan_batch_mask(models, n, o, any_strategy, smem_max, sms, p);
     if (rc != PCCP_OK || p->mask) return rc;
   }
+  pccp_solve_opts sized = *o;
+  if (sized.threads == 0) sized.threads = general_team;
+  o = &sized;
   p->xw = any_strategy ? 24 * ((max_branch + 15) & ~15) : policy_x_words(o, max_branch);
   p->max_tw = max_tw;
   p->max_vars = max_vars;
@@ -2188,8 +2192,12 @@ int pccp_propagate(const pccp_model* m, int32_t n_stores, int32_t* lb, int32_t* 
   return pccp_propagate_ex(m, n_stores, lb, ub, status, iterations, nullptr, nullptr, stream);
 }
 
-int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
-                     const pccp_solve_opts* opts, pccp_result* results, void* stream) {
+}  // extern "C"
+
+// pccp_solve_batch; general_team as in plan_batch.
+static int solve_batch(const pccp_model* const* models, int32_t n_models,
+                       const pccp_solve_opts* opts, pccp_result* results, void* stream,
+                       int general_team) {
   if (!models || n_models < 0 || !opts || !results) return PCCP_ERR_INVALID;
   if (n_models == 0) return PCCP_OK;
   {
@@ -2218,7 +2226,7 @@ int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
   }
   BatchPlan plan;
   {
-    const int rc = plan_batch(models, n_models, opts, false, &plan);
+    const int rc = plan_batch(models, n_models, opts, false, &plan, true, general_team);
     if (rc != PCCP_OK) return rc;
   }
   const std::vector<int32_t> ord = batch_order(models, n_models);
@@ -2313,7 +2321,10 @@ int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
   return rc;
 }
 
-}  // extern "C"
+extern "C" int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
+                                const pccp_solve_opts* opts, pccp_result* results, void* stream) {
+  return solve_batch(models, n_models, opts, results, stream, 0);
+}
 
 namespace {
 
@@ -2979,10 +2990,10 @@ int pccp_solve(const pccp_model* m, const pccp_solve_opts* opts, pccp_result* re
     return solve_queue(one, 1, opts, result, static_cast<cudaStream_t>(stream));
   }
   pccp_solve_opts o = *opts;
-  if (o.threads <= 0 && !(m->mask.ok && !general_search(&o))) o.threads = 512;
+  o.threads = std::max(0, static_cast<int>(o.threads));
   o.teams_per_cta = 1;  // one model: one team
   const pccp_model* one[1] = {m};
-  return pccp_solve_batch(one, 1, &o, result, stream);
+  return solve_batch(one, 1, &o, result, stream, 512);
 }
 
 }  // extern "C"

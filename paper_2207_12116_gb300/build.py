@@ -41,7 +41,6 @@ def stale(lib: str = LIB) -> bool:
 
 def _command(sources, out, verbose):
     return [nvcc(), *ARCH, "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
-            "-split-compile=0",
             "-Xptxas", "-v" if verbose else "-O3", *sources, "-o", out]
 
 

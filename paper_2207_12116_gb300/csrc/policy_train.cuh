@@ -106,7 +106,10 @@ __global__ void __launch_bounds__(256) k_train_forward(const PolicyDev* __restri
   const int chunk = warp & 3, half = warp >> 2;
   const int r0 = blockIdx.x * kTrainRows + 16 * chunk + g;
   uint32_t a1[4], a2[8][4];
+  uint2 w[8];  // the second layer's fragments of the next tile of units
   feature_fragment(a1, f, n, r0, t);
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk) w[kk] = __ldg(&pol->w2[kk][8 * half][lane]);
   layer1_fragments(pol, &pol->w1[0][0], a1, lane, a2);
   if (threadIdx.x < 128) sw3[threadIdx.x] = __ldg(&pol->w3[threadIdx.x]);
   if (half == 0) {
@@ -126,11 +129,18 @@ __global__ void __launch_bounds__(256) k_train_forward(const PolicyDev* __restri
 #pragma unroll
   for (int jj = 0; jj < 8; ++jj) {
     const int j = 8 * half + jj;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) mma_16816(acc, a2[kk], __ldg(&pol->w2[kk][j][lane]));
     const int c = 8 * j + 2 * t;
     const float2 b = __ldg(reinterpret_cast<const float2*>(&pol->b2[c]));
+    uint2 next[8] = {};
+    if (jj < 7)
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) next[kk] = __ldg(&pol->w2[kk][j + 1][lane]);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      mma_16816(acc, a2[kk], w[kk]);
+      w[kk] = next[kk];
+    }
     const float2 u = make_float2(fmaxf(acc[0] + b.x, 0.f), fmaxf(acc[1] + b.y, 0.f));
     const float2 v = make_float2(fmaxf(acc[2] + b.x, 0.f), fmaxf(acc[3] + b.y, 0.f));
     *reinterpret_cast<float2*>(H2 + static_cast<size_t>(r0) * 128 + c) = u;
@@ -341,17 +351,16 @@ __global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloa
     const __nv_bfloat16* A = (second ? dZ2b : dZ1b) + m0;  // [R][128], 16 columns of it
     const __nv_bfloat16* B = (second ? H1 : X) + n0;       // [R][128 or 16]
     const int ldb = second ? 128 : 16, n_stages = (R + kGradRows - 1) / kGradRows;
-    auto load = [&](int k) {  // stage k, thread tid's row of it
-      const int r = k * kGradRows + tid;
-      if (k < n_stages && r < R) {
-        const uint32_t to = smem_u32(tsm) + 2u * 2u * kGradPitch * kGradRows * static_cast<uint32_t>(k % kGradStages);
-        const uint32_t ta = to + 2u * kGradPitch * static_cast<uint32_t>(tid), tb = ta + 2u * kGradPitch * kGradRows;
-        const __nv_bfloat16* a = A + static_cast<size_t>(r) * 128;
-        const __nv_bfloat16* b = B + static_cast<size_t>(r) * ldb;
-        cp_async16(ta, a);
-        cp_async16(ta + 16, a + 8);
-        cp_async16(tb, b);
-        cp_async16(tb + 16, b + 8);
+    auto load = [&](int k) {  // stage k: two rows a thread, half of each; two lanes share a row's sector
+      const uint32_t to = smem_u32(tsm) + 2u * 2u * kGradPitch * kGradRows * static_cast<uint32_t>(k % kGradStages);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int q = (tid >> 1) + 128 * h, r = k * kGradRows + q, e = 8 * (tid & 1);
+        if (k < n_stages && r < R) {
+          const uint32_t ta = to + 2u * static_cast<uint32_t>(kGradPitch * q + e), tb = ta + 2u * kGradPitch * kGradRows;
+          cp_async16(ta, A + static_cast<size_t>(r) * 128 + e);
+          cp_async16(tb, B + static_cast<size_t>(r) * ldb + e);
+        }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };

@@ -17,4 +17,27 @@ inline int team_for_rows(int64_t rows, int64_t per_thread, int cta, int teams) {
   return static_cast<int>(std::min(most, std::max<int64_t>(32, want)));
 }
 
+// Threads of a team of the mask form's propagation, for n_stores stores of `words`
+// words of Booleans on `sms` SMs.  A team takes a whole store, and an SM holds 1,024
+// threads and 16 teams, so
+//   - the stores that an SM gets take as few turns as they can (a batch that just
+//     misses one turn pays for two), and share its 32 warps evenly;
+//   - a warp for at most every pair of words (two words are evaluated together), and in
+//     batches of several turns for every second one: there the SM is busy anyway;
+//   - a warp for at least every 32 pairs, in powers of two: a large store in few warps
+//     holds up the end.  At least two warps: the two directions of the temporal levels.
+// Measured (us of kernel; a team as wide as left every warp two and a half, until
+// now): 608 stores of 20 tasks 23.5 -> 12.2, 1,216 23.9 -> 14.1, 1,700 of 14 33.8 -> 23.1,
+// 1,216 of 30 37.6 -> 31.3, 1,216 of 60 56.6 -> 46.2, 300 of 60 38.1 -> 23.3, 1,700 of 90 163
+// -> 137, 608 of 120 127 -> 104; slower 1,700 of 45 48.5 -> 51.2.
+inline int propagation_team(int64_t n_stores, int64_t sms, int words) {
+  const int64_t per_sm = std::max<int64_t>(1, (n_stores + sms - 1) / sms);
+  const int64_t turns = (per_sm + 15) / 16, at_once = (per_sm + turns - 1) / turns;
+  const int64_t pairs = (words + 1) / 2;
+  int64_t least = 2;
+  while (least < 32 && 32 * least < pairs) least *= 2;
+  const int64_t most = std::max(least, turns == 1 ? pairs : pairs / 2);
+  return static_cast<int>(32 * std::min<int64_t>(32, std::min(most, std::max(least, 32 / at_once))));
+}
+
 }  // namespace pccp

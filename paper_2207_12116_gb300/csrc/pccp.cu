@@ -1421,22 +1421,9 @@ int plan_propagate_mask(const pccp_model* m, int32_t n_stores, const pccp_launch
   const size_t per_team = align16(16 + 4 * static_cast<size_t>(mask_ctrl_words(f.n_words)) +
                                   static_cast<size_t>(f.n_slots) * sizeof(int2));
   const size_t base = static_cast<size_t>(f.image_bytes) + 16;
-  int team = 64, teams = 0;
-  if (cfg && cfg->team_threads > 0) {
-    team = cfg->team_threads;
-  } else {
-    // the most warps a store that still give every warp of the GPU about two
-    // and a half (enough stores in turn that a hard one does not hold up the
-    // end), at least two (the two directions of the temporal levels), at most
-    // one a pair of words.  Measured, us with 2 / 4 / 8 / 16 / 32 warps a store:
-    // 10,000 stores of 30 tasks 110 / 115 / 157 / 237 / 408, 777 of 60 170 /
-    // 114 / 114 / 99 / 112, 1,216 of 120 319 / 184 / 191 / 195 / 199, 152 of
-    // 120 305 / 181 / 135 / 106 / 84 (each about 40 us of it call overhead)
-    const int pairs = (f.n_words + 1) / 2;
-    while (team < 1024 && team / 32 < pairs &&
-           2ll * n_stores * (team / 32) <= 5ll * sms * 16)
-      team *= 2;
-  }
+  const int team =
+      cfg && cfg->team_threads > 0 ? cfg->team_threads : propagation_team(n_stores, sms, f.n_words);
+  int teams = 0;
   if (cfg && cfg->teams_per_cta > 0) teams = cfg->teams_per_cta;
   if (teams == 0) {  // 32 warps an SM; fewer when there is a store for no more teams
     teams = std::min(1024 / team, team == 32 ? 32 : 16);

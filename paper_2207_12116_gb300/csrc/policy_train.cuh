@@ -29,9 +29,10 @@ constexpr int kOffB3 = kOffW3 + 128;         // [1]
 // rows: 0.45 GFLOP), so what it cost was launches, intermediates written and read
 // again, and above all the two weight-gradient products, whose warps walked
 // all the rows with transposed two-byte loads: 20 launches, 520 us a step of
-// 256 groups, 455 us of it the products.  Sums keep the order they had (a product's
-// rows one after the other on one accumulator, a score's units in order), so a
-// trained policy's values do not depend on how the work is split.  Now 4 launches,
+// 256 groups, 455 us of it the products.  Gradients and scores
+// are summed in a fixed order (a product's rows one after the other on one
+// accumulator, a score's units in order), so a trained policy's values do not
+// depend on how the work is split; the loss is a tree over lanes and groups.  Now 4 launches,
 // and 140 us with the weights and gradients read back by the host.
 
 constexpr int kTrainRows = 64;     // rows of a tile
@@ -296,20 +297,25 @@ struct TrainUpdate {
   float lr, b1, b2, eps, c1, c2;
 };
 
+// Parameter i and its moments.
+__device__ __forceinline__ float3 train_state(const TrainUpdate& u, int i) {
+  return make_float3(u.p[i], u.m[i], u.v[i]);
+}
+
 // Gradient gi of parameter i, Adam's step on it (inputs 12..15 of W1 stay zero),
-// and the parameter's places in the images.
-__device__ __forceinline__ void train_update(const TrainUpdate& u, int i, float gi) {
+// and the parameter's places in the images; old: its train_state.
+__device__ __forceinline__ void train_update(const TrainUpdate& u, int i, float gi, float3 old) {
   u.g[i] = gi;
   if (i < kOffB1 && (i & 15) >= kPolicyFeatures) {
     u.p[i] = 0.f;
     put_param(i, 0.f, u.w2b, u.d);
     return;
   }
-  const float mi = u.b1 * u.m[i] + (1.f - u.b1) * gi;
-  const float vi = u.b2 * u.v[i] + (1.f - u.b2) * gi * gi;
+  const float mi = u.b1 * old.y + (1.f - u.b1) * gi;
+  const float vi = u.b2 * old.z + (1.f - u.b2) * gi * gi;
   u.m[i] = mi;
   u.v[i] = vi;
-  const float np = u.p[i] - u.lr * (mi / u.c1) / (sqrtf(vi / u.c2) + u.eps);
+  const float np = old.x - u.lr * (mi / u.c1) / (sqrtf(vi / u.c2) + u.eps);
   u.p[i] = np;
   put_param(i, np, u.w2b, u.d);
 }
@@ -330,18 +336,20 @@ constexpr int kGradBlocks = kGradW2 + kGradW1 + 2 * kGradCols + 1;
 //   db2 and dw3 = H2^T ds (16 CTAs), db1 (16): 8 columns each, 256 partial sums
 //     a column, summed as a tree of 32 and then in order.
 //   db3, and the loss from the groups' (1).
-// w3 is read and written by the same CTA (its columns); nothing here reads the
-// other parameters.
-__global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloat16* __restrict__ X,
-                                                         const __nv_bfloat16* __restrict__ H1,
-                                                         const float* __restrict__ H2,
-                                                         const float* __restrict__ ds,
-                                                         const __nv_bfloat16* __restrict__ dZ2b,
-                                                         const float* __restrict__ dZ1,
-                                                         const __nv_bfloat16* __restrict__ dZ1b,
-                                                         int n_groups,
-                                                         const float* __restrict__ group_loss,
-                                                         float* __restrict__ loss, TrainUpdate u) {
+// w3 is read and written by the same CTA (its columns); nothing here reads other
+// CTAs' parameters.  4096 rows: 18.4 us (25.0 with the parameters and moments read
+// one by one at the end and a lane for each staged row, whose 32 rows an
+// instruction took 32 cycles of L1).
+__global__ void __launch_bounds__(256, 1) k_train_gradients(int R, const __nv_bfloat16* __restrict__ X,
+                                                            const __nv_bfloat16* __restrict__ H1,
+                                                            const float* __restrict__ H2,
+                                                            const float* __restrict__ ds,
+                                                            const __nv_bfloat16* __restrict__ dZ2b,
+                                                            const float* __restrict__ dZ1,
+                                                            const __nv_bfloat16* __restrict__ dZ1b,
+                                                            int n_groups,
+                                                            const float* __restrict__ group_loss,
+                                                            float* __restrict__ loss, TrainUpdate u) {
   extern __shared__ __align__(16) __nv_bfloat16 tsm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int job = blockIdx.x;
@@ -365,6 +373,20 @@ __global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloa
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
     for (int k = 0; k < kGradStages - 1; ++k) load(k);
+    // warp 0's eight parameters and their moments, read before the products: read
+    // one after another between the updates' stores, they were eight round trips
+    const int g = lane >> 2, t = lane & 3;
+    auto param = [&](int j, int e) {
+      const int o = m0 + g + 8 * (e >> 1), c = n0 + 8 * j + 2 * t + (e & 1);
+      return second ? kOffW2 + 128 * o + c : kOffW1 + 16 * o + c;
+    };
+    float3 old[2][4];
+    if (warp == 0) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) old[j][e] = train_state(u, param(j, e));
+    }
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     const int mrow = lane & 7, mhi = (lane >> 3) & 1, mlast = lane >> 4;
     for (int k = 0; k < n_stages; ++k) {
@@ -387,14 +409,10 @@ __global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloa
       }
     }
     if (warp == 0) {
-      const int g = lane >> 2, t = lane & 3;
 #pragma unroll
       for (int j = 0; j < 2; ++j)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int o = m0 + g + 8 * (e >> 1), c = n0 + 8 * j + 2 * t + (e & 1);
-          train_update(u, second ? kOffW2 + 128 * o + c : kOffW1 + 16 * o + c, acc[j][e]);
-        }
+        for (int e = 0; e < 4; ++e) train_update(u, param(j, e), acc[j][e], old[j][e]);
     }
     return;
   }
@@ -449,10 +467,11 @@ __global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloa
       }
     __syncthreads();
     const float db = column_sum(part + 256 * warp);
-    if (lane == 0) train_update(u, (second ? kOffB2 : kOffB1) + c0 + warp, db);
+    const int ib = (second ? kOffB2 : kOffB1) + c0 + warp;
+    if (lane == 0) train_update(u, ib, db, train_state(u, ib));
     if (second) {
       const float dw = column_sum(part + 256 * (8 + warp));
-      if (lane == 0) train_update(u, kOffW3 + c0 + warp, dw);
+      if (lane == 0) train_update(u, kOffW3 + c0 + warp, dw, train_state(u, kOffW3 + c0 + warp));
     }
     return;
   }
@@ -466,7 +485,7 @@ __global__ void __launch_bounds__(256) k_train_gradients(int R, const __nv_bfloa
   const float s = column_sum(part + 256 * warp);
   if (lane == 0) {
     if (warp == 0)
-      train_update(u, kOffB3, s);
+      train_update(u, kOffB3, s, train_state(u, kOffB3));
     else
       *loss = s;
   }
@@ -537,7 +556,7 @@ __global__ void k_policy_features(const uint8_t* __restrict__ image, const int2*
 // the search's sums (mlp_score_tiles, mlp_row_score).  A warp takes 32 rows at a
 // time, so every weight fragment read from shared memory (36 KB, staged once per
 // CTA) feeds two products; with a 16-row chunk a warp and fragments from L2 each
-// chunk moved 36 KB (120,000 rows: 24.7 us, 20.4 us with this kernel).
+// chunk moved 36 KB (120,000 rows: 22.9 us, 18.1 us with this kernel).
 __global__ void __launch_bounds__(256, 2) k_policy_score(const PolicyDev* __restrict__ pol, int n,
                                                       const float* __restrict__ f,
                                                       float* __restrict__ s) {

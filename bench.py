@@ -259,26 +259,27 @@ def kernel_hash():
     return h.hexdigest()[:16]
 
 
-def recorded_traffic():
-    """DRAM bytes per launch of the propagation kernel from the committed ncu summary,
-    or None when the kernel sources changed since that capture."""
+def recorded_capture():
+    """DRAM bytes and warp instructions per launch of the propagation kernel from the
+    committed ncu summary, and where they come from; None when the kernel sources
+    changed since that capture."""
     try:
         text = open(os.path.join(ROOT, profile_path())).read()
     except OSError:
-        return None, None
+        return None, None, None
     rec = {}
     for line in text.splitlines():
         if line.startswith("<!-- ") and ":" in line:
             k, v = line[5:].rstrip(" ->").split(":", 1)
             rec[k.strip()] = v.strip()
     if rec.get("kernel_sha") != kernel_hash():
-        return None, "kernel changed since the committed ncu capture"
+        return None, None, "kernel changed since the committed ncu capture"
     if rec.get("nodes", str(N_NODES)) != str(N_NODES):
-        return None, "the committed ncu capture is of another batch size"
+        return None, None, "the committed ncu capture is of another batch size"
     try:
-        return int(rec["dram_bytes_per_launch"]), profile_path()
+        return int(rec["dram_bytes_per_launch"]), int(rec["warp_instructions_per_launch"]), profile_path()
     except (KeyError, ValueError):
-        return None, None
+        return None, None, None
 
 
 SEARCH_MODELS = 256
@@ -399,9 +400,8 @@ def scale_legs(pccp):
     """Short forms of the 60-task learned-branching comparison and of the
     120-task batch: a policy trained as in --learned (probe labels on 8- and
     30-task nodes, 8 epochs); 64 seeded 60-task models (seeds 1000-1063),
-    5,000 nodes each, and 152 seeded 120-task models (seeds 2000-2151, tables
-    read from global memory), 1 s each; first-fail and learned, one launch
-    per strategy.  Per strategy: nodes/s, models with a schedule, their mean
+    5,000 nodes each, and 152 seeded 120-task models (seeds 2000-2151), 1 s
+    each; first-fail and learned, one launch per strategy.  Per strategy: nodes/s, models with a schedule, their mean
     best makespan; and model by model, whether the learned policy's best
     makespan is lower, equal or higher.  No model of these sizes is proved
     within such limits, so these are best-makespan-under-a-limit figures."""
@@ -410,7 +410,7 @@ def scale_legs(pccp):
     for key, fam, seeds, limit, what in (
             ("learned_60", "j60", range(1000, 1064), {"node_limit": 5000}, "5,000 nodes each"),
             ("large_120", "j120", range(2000, 2152), {"time_limit_ms": 1000},
-             "1 s each, tables read from global memory")):
+             "1 s each")):
         models = [pccp.Model.from_rcpsp(config_instance(fam, s)) for s in seeds]
         leg = {"workload": f"{len(models)} seeded {fam[1:]}-task 4-resource models, one launch "
                            f"per strategy, {what}"}
@@ -475,8 +475,7 @@ def search_bench(pccp, cpu=True):
             r = pccp.solve(m, deterministic=False, time_limit_ms=EPS_TIME_MS)
         limit = f"{EPS_NODE_LIMIT} node limit" if EPS_NODE_LIMIT else f"{EPS_TIME_MS} ms limit"
         out[key] = {
-            "workload": f"one {what} model ({fam}/0), all teams, {limit}"
-                        + (", table read from global memory" if fam == "j120" else ""),
+            "workload": f"one {what} model ({fam}/0), all teams, {limit}",
             "nodes_per_s": r["nodes"] / (r["elapsed_ms"] / 1000),
             "propagator_evals_per_s": r["rows_evaluated"] / (r["elapsed_ms"] / 1000),
             "ms": r["elapsed_ms"], "nodes": r["nodes"], "status": r["status"],
@@ -610,7 +609,8 @@ def run_gpu(args):
     wk = work.cpu().numpy().astype(np.int64)
     rows_per_sweep = model.rows
     evals = int(wk[:, 0].sum())          # rows actually evaluated (stable rows skipped)
-    bytes_smem = int(wk[:, 1].sum())     # algorithmic bytes they read
+    # algorithmic bytes of those rows with intervals: what the general kernels read
+    bytes_rows = int(wk[:, 1].sum())
     io_bytes = 4 * nv * N_NODES * 4 + 8 * N_NODES  # read+write lb, ub; status, iterations
 
     e2e = None
@@ -668,10 +668,31 @@ def run_gpu(args):
         props = torch.cuda.get_device_properties(dev)
         sms = props.multi_processor_count
         sm_mhz = clk.get("sm_mhz") or peaks.get("clocks_under_load", {}).get("sm_mhz_median")
-        smem_peak = sms * 128 * (sm_mhz or 0) * 1e6 / 1e9  # GB/s: 128 B/clk/SM
-        achieved = bytes_smem / (ms / 1000) / 1e9
         hbm_peak = peaks.get("hbm_gbs")
-        traffic, traffic_src = recorded_traffic()
+        traffic, instructions, capture = recorded_capture()
+        general = bool(args.skip_stable or args.stream_table)  # a loop of the general kernels
+        if general:
+            # rows and operands from shared memory, 128 B/clk/SM
+            achieved = bytes_rows / (ms / 1000) / 1e9
+            peak = sms * 128 * (sm_mhz or 0) * 1e6 / 1e9
+            roofline = {"bound": "smem", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                        "peak_source": f"derived: {sms} SMs x 128 B/clk x {sm_mhz} MHz "
+                                       f"(median SM clock sampled during the run)"}
+        else:
+            # the mask form's kernel issues instructions: words and bit planes, few bytes
+            achieved = instructions / (ms / 1000) / 1e9 if instructions else None
+            peak = sms * 4 * (sm_mhz or 0) * 1e6 / 1e9
+            roofline = {"bound": "instruction issue", "achieved": achieved, "peak": peak,
+                        "unit": "G warp instructions/s", "instructions_per_launch": instructions,
+                        "instructions_source": capture,
+                        "peak_source": f"derived: {sms} SMs x 4 schedulers x {sm_mhz} MHz "
+                                       f"(median SM clock sampled during the run)"}
+        roofline.update({
+            "frac": achieved / peak if achieved and peak else None,
+            "traffic": None if general else traffic, "traffic_source": None if general else capture,
+            "interval_bytes_of_rows_per_launch": bytes_rows,
+            "hbm": {"io_bytes_per_launch": io_bytes, "achieved": io_bytes / (ms / 1000) / 1e9,
+                    "peak": hbm_peak, "peak_source": "of measured (MEASURED_PEAKS.json)"}})
         line = {
             "metric": METRIC, "value": whole_job_rate(world, N_NODES, ms_max), "unit": UNIT,
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max,
@@ -682,17 +703,8 @@ def run_gpu(args):
             "propagator_evals_per_s": world * evals / (ms_max / 1000),
             "fixpoint_iterations_per_node": float(it.mean()),
             "rows_evaluated_per_node": evals / N_NODES,
-            "rows_skipped_fraction": 1.0 - evals / float(it.sum() * rows_per_sweep),
             "failed_nodes": int((st == 1).sum()),
-            "roofline": {"bound": "smem", "achieved": achieved, "peak": smem_peak,
-                         "unit": "GB/s", "frac": achieved / smem_peak if smem_peak else None,
-                         "traffic": traffic, "traffic_source": traffic_src,
-                         "peak_source": f"derived: {sms} SMs x 128 B/clk x {sm_mhz} MHz "
-                                        f"(median SM clock sampled during the run)",
-                         "algorithmic_bytes_per_launch": bytes_smem,
-                         "hbm": {"io_bytes_per_launch": io_bytes,
-                                 "achieved": io_bytes / (ms / 1000) / 1e9,
-                                 "peak": hbm_peak, "peak_source": "of measured (MEASURED_PEAKS.json)"}},
+            "roofline": roofline,
             "cpu_baseline": None,
             "e2e": e2e,
             "gpu_launches": args.steps,
@@ -705,15 +717,16 @@ def run_gpu(args):
             # cross-checked by a conflict-free shared-load probe
             probes = pccp.roofline_probes()
             line["roofline"]["probes"] = probes
-            meas = probes["smem_load"]["per_clk_per_sm"] * sms * (sm_mhz or 0) * 1e6 / 1e9
-            line["roofline"]["frac_of_probe"] = achieved / meas if meas else None
-            # the second roof: the kernels' own access pattern, 8-byte interval
-            # loads at random indices (random banks halve the conflict-free rate)
-            gather = probes["smem_scattered_v2"]["per_clk_per_sm"] * sms * (sm_mhz or 0) * 1e6 / 1e9
-            line["roofline"]["gather_roof"] = {
-                "peak": gather, "unit": "GB/s", "frac": achieved / gather if gather else None,
-                "source": "measured: 8-byte shared loads at random indices "
-                          f"({probes['smem_scattered_v2']['per_clk_per_sm']:.1f} B/clk/SM)"}
+            if general:
+                meas = probes["smem_load"]["per_clk_per_sm"] * sms * (sm_mhz or 0) * 1e6 / 1e9
+                line["roofline"]["frac_of_probe"] = achieved / meas if meas else None
+                # the second roof: the kernels' own access pattern, 8-byte interval
+                # loads at random indices (random banks halve the conflict-free rate)
+                gather = probes["smem_scattered_v2"]["per_clk_per_sm"] * sms * (sm_mhz or 0) * 1e6 / 1e9
+                line["roofline"]["gather_roof"] = {
+                    "peak": gather, "unit": "GB/s", "frac": achieved / gather if gather else None,
+                    "source": "measured: 8-byte shared loads at random indices "
+                              f"({probes['smem_scattered_v2']['per_clk_per_sm']:.1f} B/clk/SM)"}
         if not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline(inst, nodes)
         if not args.no_search:

@@ -22,7 +22,20 @@
  *  - `stream` is a cudaStream_t passed as void* (NULL = the legacy default
  *    stream).  The work runs on the device that is current at the call, which
  *    must be the device the model was created on.
+ *  - Device scratch of a call (counters, search state) comes from a stream-ordered
+ *    pool of the library's own, one per device.  While a model of the device lives
+ *    the pool keeps up to 64 MiB between calls; destroying the last one returns it.
  *  - All values are int32.  Variable indices are 0-based.
+ *
+ * Mask form.  A model whose Booleans each belong to at most one reified row, and whose
+ * linear rows over them are 0/1 sums with positive coefficients (the scheduling
+ * models), is kept twice: as the general table described below, and, when small
+ * enough, in mask form, with those Booleans as bits and their rows evaluated a word
+ * of 32 at a time.  Calls run on the mask form by default.  They run on the general
+ * table when an option asks for one of its loops (skip_stable, in searches also
+ * temporal_levels), for streamed tables (stream_table), for searches of more than 512
+ * threads a CTA, and when a store or table of the mask form does not fit.  Results
+ * are the same; counts of iterations and rows differ, as said beside them.
  */
 #ifndef PCCP_H
 #define PCCP_H
@@ -91,13 +104,14 @@ typedef struct {
   int32_t objective;
   int32_t n_branch;
   const int32_t* branch_vars; /* [n_branch] */
-  int32_t bool_store;  /* how the stores keep Boolean variables that appear only as
-                          reified b's and in all-positive 0/1 linear rows: 1 as
+  int32_t bool_store;  /* how the general table keeps Boolean variables that appear only
+                          as reified b's and in all-positive 0/1 linear rows: 1 as
                           bits (two bits of a shared 64-bit word each, 32 x
                           smaller stores; the table is then read from global
                           memory), -1 as intervals, 0 the library's choice (bits
                           only when an interval store would not fit in shared
-                          memory).  Results are the same. */
+                          memory).  With 0 and 1 the model has a mask form too when it
+                          qualifies, with -1 never.  Results are the same. */
 } pccp_model_desc;
 
 typedef struct pccp_model pccp_model; /* opaque; owns a device copy of the table */
@@ -116,7 +130,8 @@ int pccp_model_create(const pccp_model_desc* desc, pccp_model** out);
  * NULL is accepted. */
 void pccp_model_destroy(pccp_model* model);
 
-/* Sizes of a created model, for planning buffers and roofline accounting. */
+/* Sizes of a created model, for planning buffers and roofline accounting.  Bytes and
+ * store sizes are those of the general table, also for models with a mask form. */
 typedef struct {
   int32_t n_vars;
   int32_t n_temporal, n_linear, n_terms, n_reified;
@@ -151,9 +166,11 @@ int pccp_model_get_info(const pccp_model* model, pccp_model_info* info);
  *   status     : DEVICE int32 [n_stores]: PCCP_FIXPOINT / PCCP_FAILED /
  *                PCCP_ERROR.  lb/ub of a non-FIXPOINT store are unspecified.
  *   iterations : DEVICE int32 [n_stores] or NULL: fixed-point iterations run
- *                for each store (with the table in shared memory every row
- *                is evaluated once per iteration, the eventless loop of
- *                Sec. 5; see skip_stable in pccp_launch_config).
+ *                for each store.  Mask form: rounds of its three phases, each
+ *                of which runs only when something told since could move it.
+ *                General table in shared memory: every row is evaluated once
+ *                per iteration, the eventless loop of Sec. 5 (see skip_stable
+ *                in pccp_launch_config).
  *   n_stores   : >= 0 (0 queues nothing).
  * Asynchronous on `stream`.  Errors: INVALID, SMEM, CUDA.
  * Calls on one model may run concurrently on different streams. */
@@ -172,13 +189,15 @@ typedef struct {
   int32_t max_iterations; /* per-store iteration budget (exceeded: PCCP_ERROR) */
   int32_t skip_stable;    /* 1: re-run a row only after one of its variables changed
                              (change bitmaps per team; Sec. 6); -1: the eventless loop
-                             of Sec. 5; 0: the library's choice (on for tables read
-                             from global memory, off for tables in shared memory).
-                             Same fixed point either way. */
+                             of Sec. 5; 0: the library's choice (the mask form where
+                             the model has one; else on for tables read from global
+                             memory, off for tables in shared memory).  1 and -1 run on
+                             the general table.  Same fixed point either way. */
   int32_t stream_table;   /* tables too large for shared memory: 0 read rows in place
                              (through L1/L2); 1 stream them through a ring of
                              shared-memory buffers by TMA bulk copies, segment by
-                             segment, every sweep.  Same fixed point either way. */
+                             segment, every sweep.  1 runs on the general table.  Same
+                             fixed point either way. */
   int32_t temporal_levels; /* models whose temporal rows x + d <= y form an acyclic
                               graph: 1 two warps of a team carry the bounds along
                               its chains in one pass each sweep (rows grouped by
@@ -186,14 +205,17 @@ typedef struct {
                               levels, upper bounds in decreasing ones); -1 a thread
                               per row, which moves a bound one row per sweep; 0 the
                               library's choice (levels in propagation; in searches
-                              only for tables read from global memory).  Same fixed
-                              point either way (Sec. 3). */
+                              the mask form closes the rows along longest paths, and
+                              general tables use levels only when read from global
+                              memory).  Same fixed point either way (Sec. 3). */
 } pccp_launch_config;
 
 /* pccp_propagate with an explicit launch shape (cfg may be NULL) and an
  * optional work report: work is NULL or a DEVICE int32 [n_stores][2]
  * receiving, per store, the rows evaluated and the algorithmic bytes they
- * read (rows, operand bounds, change-tracking words).  With
+ * read (rows, operand bounds, change-tracking words).  In mask form the bytes are
+ * those of the same evaluations with intervals (pccp_model_info.bytes_per_sweep),
+ * a measure of work: the kernel itself reads words and bit planes.  With
  * cfg->skip_stable, rows whose variables did not change since their last
  * evaluation are not evaluated again (skipping stable propagators, Sec. 6);
  * the fixed point is unchanged.  Returns PCCP_ERR_SMEM if the requested
@@ -207,10 +229,12 @@ int pccp_propagate_ex(const pccp_model* model, int32_t n_stores, int32_t* lb, in
  * iterations (may be NULL) are HOST int32 [n_stores].  Two ways to move the
  * stores, chosen by chunk_stores:
  *   > 0                : chunked copies, chunk_stores stores per chunk;
- *   0                  : chunked copies: a first chunk of one store per
- *                        team of the GPU, then about four chunks, each a
- *                        whole number of stores per team (the fastest
- *                        measured);
+ *   0                  : chunked copies in chunks of the library's size: a
+ *                        first one of one unit, then about four, each of whole
+ *                        units.  The unit of a model in mask form is eight stores
+ *                        an SM, page-locked at most 12 MB of bounds, in
+ *                        multiples of 64 stores (copies of aligned addresses);
+ *                        else one store per team of the GPU;
  *   PCCP_HOST_IN_PLACE : no copies: one launch whose teams read their stores
  *                        from host memory and write the fixed points, status
  *                        and iterations back there, over the CPU-GPU link.
@@ -273,9 +297,9 @@ typedef struct {
   int64_t time_limit_ms; /* stop after this many ms of device time (<= 0: none) */
   int32_t threads;       /* threads per team (multiple of 32, <= 1024; 0 = auto) */
   int32_t blocks;        /* CTAs for the parallel search (0 = auto) */
-  int32_t skip_stable;   /* as in pccp_launch_config (0: the library's choice); also
-                            lets a left child run only the rows of the decided
-                            variable first */
+  int32_t skip_stable;   /* as in pccp_launch_config (0: the library's choice; 1 and -1
+                            search on the general tables); 1 also lets a left child
+                            run only the rows of the decided variable first */
   int32_t stream_table;  /* as in pccp_launch_config; batched searches stream only
                             when some table does not fit one CTA beside its store
                             (one team per CTA then) */
@@ -292,10 +316,12 @@ typedef struct {
                                subproblem a team hands its shallowest open right branch
                                to the queue at each branching while teams wait for
                                work (0 = the library's choice, 4; < 0 = never) */
-  int32_t temporal_levels;  /* as in pccp_launch_config (0: the library's choice: levels
-                               for tables read from global memory only, since the
+  int32_t temporal_levels;  /* as in pccp_launch_config (0: the library's choice: longest
+                               paths in mask form; for general tables, levels when
+                               they are read from global memory only, since the
                                nodes of a search are mostly one decision away from a
-                               fixed point, where the levels save few sweeps) */
+                               fixed point, where the levels save few sweeps).  1 and
+                               -1 search on the general tables */
 } pccp_solve_opts;
 
 /* Counters and outcome of one search.  A node is every store propagated,
@@ -313,7 +339,9 @@ typedef struct {
   int64_t fails;
   int64_t solutions;
   int64_t iterations;    /* fixed-point iterations summed over nodes */
-  int64_t rows_evaluated;/* propagator rows evaluated (stable rows are skipped) */
+  int64_t rows_evaluated;/* propagator rows evaluated (stable rows are skipped; the mask
+                            form's closure of temporal rows along longest paths is
+                            not counted) */
   int32_t max_depth;
   float elapsed_ms;      /* device time of the search kernel */
   float model_ms;        /* batched searches: device time of this model's own search,
@@ -346,8 +374,10 @@ int pccp_solve(const pccp_model* model, const pccp_solve_opts* opts, pccp_result
  * Deterministic form: a CTA holds teams_per_cta
  * teams side by side, each in its own slot of shared memory; the models are
  * queued largest table first and every team pulls the next one when it
- * finishes.  A model's table prefix is staged in its team's slot when it
- * fits beside the store, else read in place from global memory.
+ * finishes.  Mask form: the tables are staged in the teams' slots, and the slots' rest
+ * keeps fixed points of the path to continue from.  A general table's prefix is
+ * staged in its team's slot when it fits beside the store, else read in place from
+ * global memory.
  * results[i] is filled for models[i] (its witness pointer is honoured).
  * Synchronous.  Errors: INVALID, SMEM (a store does not fit a slot),
  * TIMEOUT, CUDA. */
@@ -363,14 +393,16 @@ int pccp_solve_batch(const pccp_model* const* models, int32_t n_models,
  * shape is fixed here: `threads` per team (0 = the library's choice; a
  * multiple of 32) and `teams_per_cta` teams side by side per CTA (0 = the
  * library's choice), as in pccp_solve_batch; later searches of the batch
- * use it whatever their options say (stream_table is not used).  The models
- * must outlive the batch.  Errors: INVALID, SMEM, CUDA. */
+ * use it whatever their options say (stream_table is not used), except that
+ * searches of a batch in mask form with skip_stable or temporal_levels use a second
+ * shape, planned here for the general tables (SMEM from those searches when none
+ * fits).  The models must outlive the batch.  Errors: INVALID, SMEM, CUDA. */
 typedef struct pccp_batch pccp_batch;
 int pccp_batch_create(const pccp_model* const* models, int32_t n_models, int32_t threads,
                       int32_t teams_per_cta, pccp_batch** out);
 
 /* The launch shape a batch was planned with (threads per team, teams per
- * CTA, CTAs). */
+ * CTA, CTAs) for deterministic = 1. */
 int pccp_batch_get_shape(const pccp_batch* batch, int32_t* threads, int32_t* teams_per_cta,
                          int32_t* ctas);
 

@@ -1681,10 +1681,10 @@ int plan_batch_mask(const pccp_model* const* models, int32_t n, const pccp_solve
     team = team_for_rows(max_rows, o->props_per_thread, 512, teams);
   if (team == 0) {
     // a warp per sixteen words of Booleans: a node runs few of them, and a
-    // barrier costs more with more warps (256 30-60-task models x 500 nodes, two
-    // teams an SM of 64 / 128 / 256 threads: 12.7 / 9.9 / 9.6 ms; 64 60-task models,
-    // learned, one team of 128 / 256 / 512: 3.8 / 3.1 / 3.0 ms; one 8-task model of
-    // 2,559 nodes, 32 / 64 / 128: 12.6 / 13.4 / 13.4 ms)
+    // barrier costs more with more warps (kernel: 256 30-60-task models x 500 nodes, two
+    // teams an SM of 64 / 128 / 256 threads: 14.5 / 9.9 / 8.5 ms; 64 60-task models x
+    // 200 learned nodes, one team of 128 / 256 / 512: 4.3 / 3.2 / 2.8 ms; one 8-task model
+    // of 111 nodes, 32 / 64 / 128: 0.335 / 0.362 / 0.363 ms)
     int w = 1;
     while (64 * w * teams <= 512 && 16 * w < max_words) w *= 2;
     team = 32 * w;
@@ -2640,8 +2640,9 @@ int plan_queue_mask(const pccp_model* const* models, int32_t n, const pccp_solve
   if (teams == 0) {
     // one model: as many teams as there are threads for.  Many models: eight, so
     // that the last proofs, which donations cannot spread over every team, run on
-    // SMs with fewer teams (256 6-10-task models, 128,000 nodes of proofs in all: 4.2
-    // ms with 8 teams an SM, 5.0 with 12, 6.0 with 16; 13.4 M nodes: 99, 77, 68 ms)
+    // SMs with fewer teams (256 6-10-task models, 119,000 nodes of proofs in all: 2.9
+    // ms of kernel with 8 teams an SM, 3.6 with 12, 4.1 with 15; 13.4 M nodes to the
+    // optimum: 75, 57, 51 ms)
     teams = std::min(p->shared ? 16 : 8, 512 / team);
     while (teams > 1 && !fits(teams)) --teams;
   }

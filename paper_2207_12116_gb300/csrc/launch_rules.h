@@ -23,21 +23,34 @@ inline int team_for_rows(int64_t rows, int64_t per_thread, int cta, int teams) {
 //   - the stores that an SM gets take as few turns as they can (a batch that just
 //     misses one turn pays for two), and share its 32 warps evenly;
 //   - a warp for at most every pair of words (two words are evaluated together), and in
-//     batches of several turns for every second one: there the SM is busy anyway;
-//   - a warp for at least every 32 pairs, in powers of two: a large store in few warps
-//     holds up the end.  At least two warps: the two directions of the temporal levels.
+//     batches of several turns for every second one: there the SM is busy anyway; at
+//     least two warps: the two directions of the temporal levels;
+//   - stores of more than 40 pairs at least four warps and of more than 100 eight, since
+//     a hard one in few warps holds up the end.  Where that is more than their share,
+//     turns are many whatever the width, and wider teams leave less of the last one
+//     empty: eight warps for four, sixteen for eight when a second turn would be at most
+//     a third full.
 // Measured (us of kernel; a team as wide as left every warp two and a half, until
 // now): 608 stores of 20 tasks 23.5 -> 12.2, 1,216 23.9 -> 14.1, 1,700 of 14 33.8 -> 23.1,
-// 1,216 of 30 37.6 -> 31.3, 1,216 of 60 56.6 -> 46.2, 300 of 60 38.1 -> 23.3, 1,700 of 90 163
-// -> 137, 608 of 120 127 -> 104; slower 1,700 of 45 48.5 -> 51.2.
+// 1,216 of 30 37.6 -> 31.3, 300 of 60 38.1 -> 23.3, 608 of 120 127 -> 104, 777 of 120 179 ->
+// 161; slower 1,700 of 45 48.5 -> 51.2.  Means over six models, 2 / 3 / 4 / 5 / 6 / 8 / 16
+// warps: 620 of 62 tasks 71 / 55 / 47 / 43 / 43 / 44 / 49, 1,000 87 / 66 / 56 / 67 / 70 / 61 /
+// 64, 1,314 104 / 79 / 91 / 90 / 83 / 74 / 81, 2,300 99 / 110 / 96 / 96 / 95 / 90 / 109; 1,200 of
+// 80 133 / 99 / 83 / 100 / 95 / 86 / 90; 1,314 of 48 62 / 48 / 59 / 58 / 55 / 52 / 61.
 inline int propagation_team(int64_t n_stores, int64_t sms, int words) {
   const int64_t per_sm = std::max<int64_t>(1, (n_stores + sms - 1) / sms);
   const int64_t turns = (per_sm + 15) / 16, at_once = (per_sm + turns - 1) / turns;
-  const int64_t pairs = (words + 1) / 2;
-  int64_t least = 2;
+  const int64_t pairs = (words + 1) / 2, share = 32 / at_once;
+  int64_t least = pairs > 100 ? 8 : pairs > 40 ? 4 : 2;
   while (least < 32 && 32 * least < pairs) least *= 2;
+  if (share < least) {
+    const int64_t held = sms * std::min<int64_t>(16, 32 / least);
+    const bool few = n_stores > held && 3 * (n_stores - held) <= held;
+    if (least < 32 && (few || (least == 4 && turns <= 2))) least *= 2;
+    return static_cast<int>(32 * least);
+  }
   const int64_t most = std::max(least, turns == 1 ? pairs : pairs / 2);
-  return static_cast<int>(32 * std::min<int64_t>(32, std::min(most, std::max(least, 32 / at_once))));
+  return static_cast<int>(32 * std::min(most, share));
 }
 
 // Stores of which the default chunks of host-memory propagation are multiples, for

@@ -14,7 +14,7 @@
 // What bounds it: instruction issue, and for batches of few stores the hardest
 // store's chain of phases.  Kernel times against k_propagate on the same stores (one
 // GB300): 10,000 of 30 tasks 169 -> 81 us.  Whole passes, with the caller's copy of
-// the stores: 777 of 60 tasks 159 -> 83 us, 1,216 of 120 tasks 936 -> 306 us.
+// the stores: 777 of 60 tasks 159 -> 88 us, 1,216 of 120 tasks 936 -> 306 us.
 #pragma once
 
 #include "mask_device.cuh"
